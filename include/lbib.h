@@ -390,7 +390,8 @@ int lbib_label_cells(int32_t nx, int32_t ny, int32_t bc_y, int32_t n_cells,
  *   d_workspace, ws_bytes  device scratch of lbib_steady_workspace_size()
  *               bytes, 256-byte aligned, owned by the caller
  * FP32 storage and arithmetic.  Synchronises the stream.  Returns LBIB_OK,
- * LBIB_E_PARAM, LBIB_E_WORKSPACE or LBIB_E_CUDA. */
+ * LBIB_E_PARAM, LBIB_E_WORKSPACE or LBIB_E_CUDA. LBIB_E_TIMEOUT: a
+ * wait between the CTAs that share a tissue ran out (about a second). */
 int lbib_steady_workspace_size(int32_t nx, int32_t ny, int32_t batch, uint64_t* bytes_out);
 int lbib_steady_solve(int32_t nx, int32_t ny, int32_t batch, const uint8_t* d_src,
                       const double* D, const double* decay, const double* src_rate,
