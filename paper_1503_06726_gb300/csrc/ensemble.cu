@@ -127,7 +127,7 @@ __device__ __forceinline__ int find_tissue(const int* pfx, int n, int item) {
 __host__ __device__ inline int ens_cell_threads(int maxv) { return maxv <= 64 ? 64 : 128; }
 
 __host__ __device__ inline size_t ens_cell_smem(int maxv) {
-    return (size_t)kIBSmemFixed + (size_t)maxv * kIBSmemPerVertex;
+    return ((size_t)kIBSmemFixed + (size_t)maxv * kIBSmemPerVertex + 15) / 16 * 16;
 }
 
 template <int S, int FORCING>

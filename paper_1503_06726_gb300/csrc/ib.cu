@@ -24,6 +24,7 @@
 #include <type_traits>
 
 #include "ib_cell.cuh"
+#include "ib_cell_half.cuh"
 
 namespace lbib {
 
@@ -242,11 +243,26 @@ __global__ void __launch_bounds__(NT) ib_cell_kernel_f32(IBArgs a, int maxv) {
     ib_f32_body<NT>(a, maxv);
 }
 
-// the 64-thread kernel (many small cells) held to 56 registers, 18 CTAs per
-// SM instead of 16 at its natural 64: more cells in flight for a
-// latency-bound launch (C3, 9,801 cells: 107.7 -> 104.6 us)
-__global__ void __launch_bounds__(64, 18) ib_cell_kernel_f32_64(IBArgs a, int maxv) {
+// the 64-thread kernel (many small cells): 12 CTAs per SM leave it the 80
+// registers that hold a vertex's velocity rows at once (9,801 cells: 79 us;
+// 81 at 14 or 16 CTAs, 82 at 10, 123 at 20, where the rows spill)
+__global__ void __launch_bounds__(64, 12) ib_cell_kernel_f32_64(IBArgs a, int maxv) {
     ib_f32_body<64>(a, maxv);
+}
+
+// FP16 storage: the same kernels over ib_cell_half
+template <int NT>
+__device__ __forceinline__ void ib_half_body(const IBArgs& a, int maxv) {
+    extern __shared__ __align__(16) unsigned char ib_smem[];
+    const IBSharedHalf S = ib_shared_half_view(ib_smem, maxv);
+    ib_cell_half<NT>(a, blockIdx.x, S, threadIdx.x, 0);
+}
+template <int NT>
+__global__ void __launch_bounds__(NT) ib_cell_kernel_half(IBArgs a, int maxv) {
+    ib_half_body<NT>(a, maxv);
+}
+__global__ void __launch_bounds__(64, 18) ib_cell_kernel_half_64(IBArgs a, int maxv) {
+    ib_half_body<64>(a, maxv);
 }
 
 cudaError_t launch_ib(int precision, const IBArgs& a, int maxv_cell, cudaStream_t s, bool pdl) {
@@ -258,6 +274,17 @@ cudaError_t launch_ib(int precision, const IBArgs& a, int maxv_cell, cudaStream_
     // largest cell let many more CTAs be resident per SM
     int maxv = maxv_cell < 3 ? 3 : (maxv_cell > kMaxVertsPerCell ? kMaxVertsPerCell : maxv_cell);
     maxv = (maxv + 7) / 8 * 8;
+    if (precision == LBIB_FP16) {
+        const size_t half = kIBSmemHalfFixed + (size_t)maxv * kIBSmemHalfPerVertex;
+        if (maxv <= 64 && a.n_cells >= 2048)
+            return launch_kernel(ib_cell_kernel_half_64, dim3(a.n_cells), dim3(64), half, s, pdl,
+                                 a, maxv);
+        if (maxv <= 128 && a.n_cells >= 2048)
+            return launch_kernel(ib_cell_kernel_half<128>, dim3(a.n_cells), dim3(128), half, s,
+                                 pdl, a, maxv);
+        return launch_kernel(ib_cell_kernel_half<256>, dim3(a.n_cells), dim3(256), half, s, pdl,
+                             a, maxv);
+    }
     const size_t smem = kIBSmemFixed + (size_t)maxv * kIBSmemPerVertex;
     if (maxv <= 64 && a.n_cells >= 2048)
         return launch_kernel(ib_cell_kernel_f32_64, dim3(a.n_cells), dim3(64), smem, s, pdl, a,

@@ -18,6 +18,11 @@ __device__ __forceinline__ int wrapi(int a, int n) {
     return r < 0 ? r + n : r;
 }
 
+// the same for an index that mostly lies in [0, n): no division there
+__device__ __forceinline__ int wrap_near(int a, int n) {
+    return (unsigned)a < (unsigned)n ? a : wrapi(a, n);
+}
+
 // Weights of the 4 support nodes along one axis, base = floor(X) - 1.
 // With f = X - floor(X) the four offsets are r = -1-f, -f, 1-f, 2-f, and
 // cos(pi |r| / 2) is -sin, cos, sin, -cos of pi f / 2 respectively, so one
@@ -193,43 +198,49 @@ __device__ __forceinline__ void mark_row(const IBArgs& a, uint32_t* mask, int64_
     if (LBIB_CHK_INDEX(a.diag, kSiteMask, wd, mask_words(a.plane))) atomicOr(mask + wd, bits);
 }
 
-// OR `bits` into mask word `wd` through the CTA's table of the cell's words
-// (open addressing in shared memory; the word goes to the mask once, at the
-// flush after the spreading); a full table falls back to the global atomic.
-__device__ __forceinline__ void mask_or_table(const IBArgs& a, uint32_t* mask, int64_t wd,
-                                              uint32_t bits, uint32_t* mkey, uint32_t* mval) {
-    if (!LBIB_CHK_INDEX(a.diag, kSiteMask, wd, mask_words(a.plane))) return;
-    const uint32_t k = (uint32_t)wd;
-    uint32_t h = (k * 2654435761u) >> (32 - kMaskTableLog2);
-#pragma unroll 1
-    for (int probe = 0; probe < 16; ++probe) {
-        const uint32_t old = atomicCAS(mkey + h, kMaskEmpty, k);
-        if (old == kMaskEmpty || old == k) {
-            atomicOr(mval + h, bits);
-            return;
-        }
-        h = (h + 1) & (uint32_t)(kMaskTable - 1);
-    }
-    atomicOr(mask + wd, bits);
+// The force-mask groups of one cell, one byte per 4-node group of the box of
+// its stencils (rows of kGroupCols groups): marked with plain byte stores,
+// which need no atomics, then ORed into the mask row by row.  The box of a
+// cell that is too large or crosses the periodic seam in x does not fit; its
+// vertices mark the mask themselves.
+struct GroupBox {
+    bool fits;
+    int row0;   // unwrapped row of the first table row
+    int rows;
+    int g0;     // in-row group of the first column
+};
+__device__ __forceinline__ GroupBox group_box(const IBArgs& a, int ilo, int ihi, int jlo, int jhi) {
+    // stencils cover the columns ilo - 1 .. ihi + 2 and, with jlo and jhi the
+    // ends of ceil(y), rows within jlo - 2 .. jhi + 2
+    GroupBox g;
+    const int xa = wrap_near(ilo - 1, a.nx), w = ihi - ilo + 4;
+    g.row0 = jlo - 2;
+    g.rows = jhi - jlo + 5;
+    g.g0 = xa >> 2;
+    g.fits = a.fmask != nullptr && w <= a.nx - xa && ((xa + w - 1) >> 2) - g.g0 < kGroupCols &&
+             g.rows <= kGroupRows;
+    return g;
 }
-
-// mark_row through the table
-__device__ __forceinline__ void mark_row_table(const IBArgs& a, uint32_t* mask, int64_t rowbase,
-                                               const int ix[4], uint32_t* mkey, uint32_t* mval) {
-    if (!mask) return;
-    int64_t wd = -1;
-    uint32_t bits = 0u;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int64_t g = (rowbase + ix[i]) >> 2;
-        if ((g >> 5) != wd) {
-            if (bits) mask_or_table(a, mask, wd, bits, mkey, mval);
-            wd = g >> 5;
-            bits = 0u;
-        }
-        bits |= 1u << (g & 31);
+// every marked group of the cell into the mask, one thread per row
+template <int NT>
+__device__ __forceinline__ void flush_groups(const IBArgs& a, const GroupBox& g,
+                                             const uint8_t* table, int tid) {
+    for (int r = tid; r < g.rows; r += NT) {
+        const uint4 v = reinterpret_cast<const uint4*>(table)[r];
+        if ((v.x | v.y | v.z | v.w) == 0u) continue;
+        // bytes of 0 or 1 to bits: the products' bits never meet
+        const uint32_t bits = (v.x * 0x10204080u >> 28) | (v.y * 0x10204080u >> 28) << 4 |
+                              (v.z * 0x10204080u >> 28) << 8 | (v.w * 0x10204080u >> 28) << 12;
+        // (marked rows lie inside a walled lattice: row0 + r is in [0, ny))
+        const int J = a.bc_y ? g.row0 + r : wrap_near(g.row0 + r, a.ny);
+        const int grp = ((J * (int)a.pitch) >> 2) + g.g0;
+        const unsigned long long m = (unsigned long long)bits << (grp & 31);
+        const int w = grp >> 5;
+        if ((uint32_t)m && LBIB_CHK_INDEX(a.diag, kSiteMask, w, mask_words(a.plane)))
+            atomicOr(a.fmask + w, (uint32_t)m);
+        if ((uint32_t)(m >> 32) && LBIB_CHK_INDEX(a.diag, kSiteMask, w + 1, mask_words(a.plane)))
+            atomicOr(a.fmask + w + 1, (uint32_t)(m >> 32));
     }
-    mask_or_table(a, mask, wd, bits, mkey, mval);
 }
 
 // Mark the groups of the nodes [s, e) of one row (no wrap inside the range)
@@ -514,12 +525,11 @@ __device__ __forceinline__ float2 edge_vec(int2 ba, float2 fa, int2 bb, float2 f
     return make_float2((float)(bb.x - ba.x) + (fb.x - fa.x), (float)(bb.y - ba.y) + (fb.y - fa.y));
 }
 
-// spring force on the first vertex of an edge with vector d (FP32)
-__device__ __forceinline__ float2 spring32(float2 d, float L0, float kk) {
+// spring force on the first vertex of an edge with vector d (FP32), over d
+__device__ __forceinline__ float spring32(float2 d, float L0, float kk) {
     const float len2 = d.x * d.x + d.y * d.y;
     const float len = sqrtf(len2);
-    const float sc = kk * ((len2 - L0 * L0) / (len + L0)) / len;
-    return make_float2(sc * d.x, sc * d.y);
+    return kk * ((len2 - L0 * L0) / (len + L0)) / len;
 }
 
 // The work of one cell by NT threads (thread index tid, barrier bar: the
@@ -534,27 +544,30 @@ __device__ __forceinline__ float2 spring32(float2 d, float L0, float kk) {
 // out of line (the small-CTA kernels keep few registers, 18 CTAs of 64
 // threads per SM, and the ensemble's persistent kernel its budget)
 // OPTS = false compiles out the junction forces and mass sources (the
-// ensemble has neither).  The force-mask bits go through the cell slot's
-// table of mask words (one global OR per distinct word instead of one per
-// vertex and stencil row: the small-CTA kernels of many cells, whose ORs to
-// shared words throttle the launch; 4096^2, 9,801 cells: IB launch 104 -> 93
-// us), or straight to the mask (the 256-thread kernel of few large cells,
-// where the table's extra barrier lengthens each cell's chain: 1024^2, 400
-// cells, 16.7 -> 22 us with it).
+// ensemble has neither).
+// A cell's time is the latency of its few dependent accesses times the warps
+// that share an SM, so the work per access is kept small and the accesses
+// wide: all velocity rows of a vertex are loaded before any is used (1024^2,
+// 400 cells: 17.9 -> 15.6 us), an index is divided by the lattice size only
+// when it lies outside it, an edge's spring is computed once for both its
+// vertices, and the force-mask groups are marked with plain bytes in shared
+// memory (GroupBox).  1,268 instructions per warp of a 64-vertex cell in place
+// of 4,900; 4096^2, 9,801 cells: 95.6 -> 79 us.  Sixteen lanes per vertex in
+// the spreading (fewer lines per reduction) measured the same there and 1 us
+// slower at 1024^2.
 template <int NT, bool GRIDDEP, bool INLINE_FILL = true, bool OPTS = true,
-          bool MASK_TABLE = (NT <= 128)>
+          bool GROUPS = true>
 static __device__ void ib_cell_f32(const IBArgs& a, int c, const IBShared32& S, int tid,
                                    int bar) {
     static_assert(NT % 64 == 0, "CTA size");
-    constexpr int kIBThreads = NT;
+    constexpr int NW = NT / 32;
     double2* sx = S.sx;
     int2* sb = S.sb;
     float2* sf = S.sf;
     int* rowcnt = S.rowcnt;
     int* thr = S.thr;
-    int* sbox = S.sbox;
     int& s_flag = *S.s_flag;
-    cell_sync<NT>(bar);
+    if (!GRIDDEP) cell_sync<NT>(bar);  // a kernel of its own runs one cell per CTA
 
     const int v0 = __ldcg(a.off + c);
     const int n = __ldcg(a.off + c + 1) - v0;
@@ -572,44 +585,30 @@ static __device__ void ib_cell_f32(const IBArgs& a, int c, const IBShared32& S, 
         return;
     }
 
-    for (int r = tid; r < kMaxRows; r += NT) rowcnt[r] = 0;
-    if (MASK_TABLE) {
-        for (int i = tid; i < kMaskTable; i += NT) {
-            S.mkey[i] = kMaskEmpty;
-            S.mval[i] = 0u;
-        }
-    }
-    if (tid == 0) {
-        sbox[0] = INT_MAX; sbox[1] = INT_MIN; sbox[2] = INT_MAX; sbox[3] = INT_MIN;
-        s_flag = 0;
-    }
+    // the cell is labelled when the caller wants the packed labels or the cell
+    // has source bits to deposit
+    const bool may_label =
+        a.do_prep && a.do_mask && (a.do_ids || (a.src && (__ldcg(a.srcf + c) & 0xF)));
+    if (may_label)
+        for (int r = tid; r < kMaxRows; r += NT) rowcnt[r] = 0;
+    if (GROUPS && a.do_prep && a.do_force)
+        for (int i = tid; i < kGroupRows * kGroupCols / 16; i += NT)
+            reinterpret_cast<uint4*>(S.grp)[i] = make_uint4(0u, 0u, 0u, 0u);
+    if (tid == 0) s_flag = 0;
 
-    // spring data of the vertices this thread will handle in phase 2, loaded
-    // now so that phase 2 waits on no load: vertex tid (every thread: the whole
-    // CTA computes forces when the cell is not labelled) and vertex tid + half
-    // (the first half, which alone computes forces while the second half
-    // scans the rows of a labelled cell)
-    constexpr int half = kIBThreads / 2;
-    float pL0[2] = {0.f, 0.f}, pk[2] = {0.f, 0.f}, pL0p[2] = {0.f, 0.f}, pkp[2] = {0.f, 0.f};
-    float ppres = 0.f;
-    if (a.do_prep && a.do_force) {
-        ppres = (float)__ldcg(a.pres + c);
-#pragma unroll
-        for (int r = 0; r < 2; ++r) {
-            const int t = tid + r * half;
-            if (t < n && (r == 0 || tid < half)) {
-                const int tp = (t == 0) ? n - 1 : t - 1;
-                pL0[r] = (float)__ldcg(a.L0 + v0 + t);
-                pk[r] = (float)__ldcg(a.k + v0 + t);
-                pL0p[r] = (float)__ldcg(a.L0 + v0 + tp);
-                pkp[r] = (float)__ldcg(a.k + v0 + tp);
-            }
-        }
-    }
-    // the vertex state of this thread's first vertex
+    // spring data of the edge this thread computes first, and the vertex state
+    // of its first vertex, loaded now so that nothing below waits on them
+    float pL0 = 0.f, pk = 0.f, ppres = 0.f;
     double2 X0 = make_double2(0.0, 0.0);
     int2 b0 = make_int2(0, 0);
     float2 f0 = make_float2(0.f, 0.f);
+    if (a.do_prep && a.do_force) {
+        ppres = (float)__ldcg(a.pres + c);
+        if (tid < n) {
+            pL0 = (float)__ldcg(a.L0 + v0 + tid);
+            pk = (float)__ldcg(a.k + v0 + tid);
+        }
+    }
     if (tid < n) {
         X0 = __ldcg(a.xy + v0 + tid);
         if (a.do_move && a.vbase) {
@@ -621,11 +620,12 @@ static __device__ void ib_cell_f32(const IBArgs& a, int c, const IBShared32& S, 
         griddep_wait();
         griddep_launch_dependents();
     }
+    const int pitch = (int)a.pitch;  // a plane holds fewer than 2^31 nodes
 
     // ---- (1) interpolate u^n at X^n and move; (base, frac) of the new X
     int ilo = INT_MAX, ihi = INT_MIN, jlo = INT_MAX, jhi = INT_MIN;
     bool finite = true;
-    for (int t = tid; t < n; t += kIBThreads) {
+    for (int t = tid; t < n; t += NT) {
         double2 X = (t == tid) ? X0 : a.xy[v0 + t];
         int2 b;
         float2 f;
@@ -642,46 +642,64 @@ static __device__ void ib_cell_f32(const IBArgs& a, int c, const IBShared32& S, 
             weights_from_frac(f.y, wy);
             const float2* u = static_cast<const float2*>(a.u);
             float Ux = 0.f, Uy = 0.f;
-            int ix[4];
-            ix[0] = wrapi(b.x - 1, a.nx);
+            const int x0 = wrap_near(b.x - 1, a.nx);
+            const bool seam = x0 + 3 >= a.nx, odd = x0 & 1;
+            int rb[4];  // the rows' first nodes, < 0 outside a walled lattice
+            {
+                int J = a.bc_y ? b.y - 1 : wrap_near(b.y - 1, a.ny);
 #pragma unroll
-            for (int i = 1; i < 4; ++i) ix[i] = (ix[i - 1] + 1 == a.nx) ? 0 : ix[i - 1] + 1;
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                int J = b.y - 1 + j;
-                if (a.bc_y) {
-                    if (J < 0 || J >= a.ny) continue;
-                } else {
-                    J = wrapi(J, a.ny);
+                for (int j = 0; j < 4; ++j, ++J) {
+                    if (!a.bc_y && J >= a.ny) J -= a.ny;
+                    rb[j] = (unsigned)J < (unsigned)a.ny ? J * pitch : -1;
                 }
-                const float2* row = u + (int64_t)J * a.pitch;
-                // the four nodes of the row, 16 bytes per load where aligned
-                float2 v[4];
-                if (ix[3] == ix[0] + 3) {
-                    const float2* r0 = row + ix[0];
-                    if ((ix[0] & 1) == 0) {
-                        const float4 p0 = u_ld4(a, r0);
-                        const float4 p1 = u_ld4(a, r0 + 2);
-                        v[0] = make_float2(p0.x, p0.y);
-                        v[1] = make_float2(p0.z, p0.w);
-                        v[2] = make_float2(p1.x, p1.y);
-                        v[3] = make_float2(p1.z, p1.w);
-                    } else {
-                        const float4 p1 = u_ld4(a, r0 + 1);
-                        v[0] = u_ld(a, r0);
-                        v[1] = make_float2(p1.x, p1.y);
-                        v[2] = make_float2(p1.z, p1.w);
-                        v[3] = u_ld(a, r0 + 3);
+            }
+            if (!seam) {
+                // a row's four nodes are two aligned 16-byte loads when it
+                // starts on an even node, three (one node too many at either
+                // end) when it starts on an odd one; every load before any use
+                const float2* r0 = u + (x0 - (odd ? 1 : 0));
+                float4 p[4][3];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    p[j][0] = p[j][1] = p[j][2] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (rb[j] >= 0) {
+                        p[j][0] = u_ld4(a, r0 + rb[j]);
+                        p[j][1] = u_ld4(a, r0 + rb[j] + 2);
+                        if (odd) p[j][2] = u_ld4(a, r0 + rb[j] + 4);
                     }
-                } else {
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) v[i] = u_ld(a, row + ix[i]);
                 }
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const float w = wx[i] * wy[j];
-                    Ux += v[i].x * w;
-                    Uy += v[i].y * w;
+                for (int j = 0; j < 4; ++j) {
+                    if (rb[j] < 0) continue;
+                    float2 v[4];
+                    v[0] = odd ? make_float2(p[j][0].z, p[j][0].w)
+                               : make_float2(p[j][0].x, p[j][0].y);
+                    v[1] = odd ? make_float2(p[j][1].x, p[j][1].y)
+                               : make_float2(p[j][0].z, p[j][0].w);
+                    v[2] = odd ? make_float2(p[j][1].z, p[j][1].w)
+                               : make_float2(p[j][1].x, p[j][1].y);
+                    v[3] = odd ? make_float2(p[j][2].x, p[j][2].y)
+                               : make_float2(p[j][1].z, p[j][1].w);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const float w = wx[i] * wy[j];
+                        Ux += v[i].x * w;
+                        Uy += v[i].y * w;
+                    }
+                }
+            } else {
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    if (rb[j] < 0) continue;
+                    const float wyj = wy[j];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const float2 v =
+                            u_ld(a, u + rb[j] + (x0 + i >= a.nx ? x0 + i - a.nx : x0 + i));
+                        const float w = wx[i] * wyj;
+                        Ux += v.x * w;
+                        Uy += v.y * w;
+                    }
                 }
             }
             X.x += (double)Ux;
@@ -711,15 +729,18 @@ static __device__ void ib_cell_f32(const IBArgs& a, int c, const IBShared32& S, 
     jlo = __reduce_min_sync(0xffffffffu, jlo);
     jhi = __reduce_max_sync(0xffffffffu, jhi);
     finite = __all_sync(0xffffffffu, finite);
+    // the warps' boxes side by side, a non-finite one as the whole range
+    if (lane == 0) S.wbox[tid >> 5] = make_int4(ilo, finite ? ihi : INT_MAX, jlo, jhi);
     cell_sync<NT>(bar);
-    if (lane == 0) {
-        atomicMin(&sbox[0], ilo);
-        atomicMax(&sbox[1], ihi);
-        atomicMin(&sbox[2], jlo);
-        atomicMax(&sbox[3], jhi);
-        if (!finite) s_flag = 2;
+#pragma unroll
+    for (int w = 0; w < NW; ++w) {
+        const int4 o = S.wbox[w];
+        ilo = min(ilo, o.x);
+        ihi = max(ihi, o.y);
+        jlo = min(jlo, o.z);
+        jhi = max(jhi, o.w);
     }
-    cell_sync<NT>(bar);
+    finite = ihi != INT_MAX;
     if (OPTS && a.msrc_out && tid < 32) {
         // mass source of the cell (Sec. 3.2.3): S_c = rate + alpha (A0 - A_c),
         // A_c the shoelace area of the moved polygon about its first vertex
@@ -729,107 +750,31 @@ static __device__ void ib_cell_f32(const IBArgs& a, int c, const IBShared32& S, 
     // columns: floor(x) over the vertices, widened by one on each side (the
     // fractions are FP32); rows: every J with min ceil(y) <= J < max ceil(y),
     // exactly the rows some edge crosses
-    const int I0 = sbox[0] - 1, I1 = sbox[1] + 1, J0 = sbox[2], J1 = sbox[3] - 1;
+    const int I0 = ilo - 1, I1 = ihi + 1, J0 = jlo, J1 = jhi - 1;
     // a box no wider than the lattice keeps the wrapped indices of the fill
     // within one period; anything wider means the geometry has blown up
-    const bool geom_ok = s_flag == 0 && (I1 - I0) < a.nx && (J1 - J0) <= a.ny;
+    const bool geom_ok = finite && (I1 - I0) < a.nx && (J1 - J0) <= a.ny;
     if (a.do_mask && !geom_ok && tid == 0) raise_flag(a.diag, kDiagGeometry);
-    // the cell is labelled when the caller wants the packed labels or the cell
-    // has source bits to deposit
-    const bool labels =
-        a.do_mask && geom_ok && J1 >= J0 && (a.do_ids || (a.src && (a.srcf[c] & 0xF)));
+    const bool labels = may_label && geom_ok && J1 >= J0;
     const int rows = J1 - J0 + 1, cols = I1 - I0 + 1;
     const bool scan = labels && rows <= kMaxRows;
-
-    if (tid < half || !scan) {  // forces: the first half, or all threads without a scan
+    GroupBox gb = {false, 0, 0, 0};
+    if (GROUPS && a.do_force && geom_ok) gb = group_box(a, ilo, ihi, jlo, jhi);
+    // the scale of every edge's spring, once (a vertex takes those of its two
+    // edges), by the first half of the threads beside the second half's
+    // scanline crossings when the cell is labelled
+    constexpr int half = NT / 2;
+    if (tid < half || !scan) {
         if (a.do_force) {
-            float2* force = static_cast<float2*>(a.force);
-            const float p = ppres;
-            const float ten = (float)a.tension;
-            const int stride = scan ? half : kIBThreads;
-            for (int t = tid, r = 0; t < n; t += stride, ++r) {
-                const int tp = (t == 0) ? n - 1 : t - 1;
+            for (int t = tid; t < n; t += scan ? half : NT) {
                 const int tn = (t == n - 1) ? 0 : t + 1;
-                const int2 b = sb[t];
-                const float2 f = sf[t];
-                const float2 dn = edge_vec(b, f, sb[tn], sf[tn]);   // X_{t+1} - X_t
-                const float2 dp = edge_vec(sb[tp], sf[tp], b, f);   // X_t - X_{t-1}
-                // prefetched for the first two vertices of this thread
-                const bool pre1 = r == 1 && stride == half;  // tid + half, prefetched
-                const float L0t = r == 0 ? pL0[0] : (pre1 ? pL0[1] : (float)a.L0[v0 + t]);
-                const float kt = r == 0 ? pk[0] : (pre1 ? pk[1] : (float)a.k[v0 + t]);
-                const float L0p = r == 0 ? pL0p[0] : (pre1 ? pL0p[1] : (float)a.L0[v0 + tp]);
-                const float kp = r == 0 ? pkp[0] : (pre1 ? pkp[1] : (float)a.k[v0 + tp]);
-                const float2 s0 = spring32(dn, L0t, kt);
-                const float2 s1 = spring32(dp, L0p, kp);
-                float Fx = s0.x - s1.x, Fy = s0.y - s1.y;
-                // pressure p dA/dX: (p/2)(y_{t+1} - y_{t-1}, x_{t-1} - x_{t+1})
-                Fx += 0.5f * p * (dn.y + dp.y);
-                Fy -= 0.5f * p * (dn.x + dp.x);
-                if (ten != 0.f) {  // Eq. membraneforce
-                    const float ln = sqrtf(dn.x * dn.x + dn.y * dn.y);
-                    const float lp = sqrtf(dp.x * dp.x + dp.y * dp.y);
-                    Fx += ten * (dn.x / ln - dp.x / lp);
-                    Fy += ten * (dn.y / ln - dp.y / lp);
-                }
-                if (OPTS && a.jpartner) {  // Eq. celljunctionforce (a launch without the move)
-                    const float2 J = junction_force32(a, sx[t], a.jpartner[v0 + t]);
-                    Fx += J.x;
-                    Fy += J.y;
-                }
-                if (a.write_vforce) a.vforce[v0 + t] = make_double2((double)Fx, (double)Fy);
-
-                float wx[4], wy[4];
-                weights_from_frac(f.x, wx);
-                weights_from_frac(f.y, wy);
-                int ix[4];
-                ix[0] = wrapi(b.x - 1, a.nx);
-#pragma unroll
-                for (int i = 1; i < 4; ++i) ix[i] = (ix[i - 1] + 1 == a.nx) ? 0 : ix[i - 1] + 1;
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    int J = b.y - 1 + j;
-                    if (a.bc_y) {
-                        if (J < 0 || J >= a.ny) {
-                            raise_flag(a.diag, kDiagWallStencil);
-                            continue;
-                        }
-                    } else {
-                        J = wrapi(J, a.ny);
-                    }
-                    float2* row = force + (int64_t)J * a.pitch;
-                    float cx4[4], cy4[4];
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const float w = wx[i] * wy[j];
-                        cx4[i] = Fx * w;
-                        cy4[i] = Fy * w;
-                    }
-                    // the four nodes of the row: two 16-byte reductions when
-                    // the row starts on an even node, 8 + 16 + 8 bytes when it
-                    // starts on an odd one, one per node across the periodic seam
-                    if (ix[3] == ix[0] + 3) {
-                        float2* r0 = row + ix[0];
-                        if ((ix[0] & 1) == 0) {
-                            force_red2(a, r0, cx4[0], cy4[0], cx4[1], cy4[1]);
-                            force_red2(a, r0 + 2, cx4[2], cy4[2], cx4[3], cy4[3]);
-                        } else {
-                            force_red1(a, r0, cx4[0], cy4[0]);
-                            force_red2(a, r0 + 1, cx4[1], cy4[1], cx4[2], cy4[2]);
-                            force_red1(a, r0 + 3, cx4[3], cy4[3]);
-                        }
-                    } else {
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) spread_add(a, &row[ix[i]], cx4[i], cy4[i]);
-                    }
-                    if (MASK_TABLE)
-                        mark_row_table(a, a.fmask, (int64_t)J * a.pitch, ix, S.mkey, S.mval);
-                    else
-                        mark_row(a, a.fmask, (int64_t)J * a.pitch, ix);
-                }
+                const bool first = t == tid;
+                S.spr[t] =
+                    spring32(edge_vec(sb[t], sf[t], sb[tn], sf[tn]),
+                             first ? pL0 : (float)a.L0[v0 + t], first ? pk : (float)a.k[v0 + t]);
             }
         }
-    } else if (scan) {
+    } else {
         for (int e = tid - half; e < n; e += half) {
             const int eb = (e == n - 1) ? 0 : e + 1;
             const int2 ba = sb[e], bb = sb[eb];
@@ -862,22 +807,111 @@ static __device__ void ib_cell_f32(const IBArgs& a, int c, const IBShared32& S, 
             }
         }
     }
-    // every distinct force-mask word of the cell into the mask, once
-    if (MASK_TABLE && a.do_force && a.fmask) {
-        cell_sync<NT>(bar);
-        for (int i = tid; i < kMaskTable; i += NT) {
-            const uint32_t k = S.mkey[i];
-            if (k != kMaskEmpty) atomicOr(a.fmask + k, S.mval[i]);
+    cell_sync<NT>(bar);
+
+    // forces and spreading: the first half of the threads in a labelled cell
+    // (the second half goes on to its rows of the label fill), else all
+    if (a.do_force && (tid < half || !scan)) {
+        float2* force = static_cast<float2*>(a.force);
+        const float hp = 0.5f * ppres;
+        const float ten = (float)a.tension;
+        for (int t = tid; t < n; t += scan ? half : NT) {
+            const int tp = (t == 0) ? n - 1 : t - 1;
+            const int tn = (t == n - 1) ? 0 : t + 1;
+            const int2 b = sb[t];
+            const float2 f = sf[t];
+            const float2 dn = edge_vec(b, f, sb[tn], sf[tn]);   // X_{t+1} - X_t
+            const float2 dp = edge_vec(sb[tp], sf[tp], b, f);   // X_t - X_{t-1}
+            const float s0 = S.spr[t], s1 = S.spr[tp];
+            const float2 e0 = make_float2(s0 * dn.x, s0 * dn.y);
+            const float2 e1 = make_float2(s1 * dp.x, s1 * dp.y);
+            float Fx = e0.x - e1.x, Fy = e0.y - e1.y;
+            // pressure p dA/dX: (p/2)(y_{t+1} - y_{t-1}, x_{t-1} - x_{t+1})
+            Fx += hp * (dn.y + dp.y);
+            Fy -= hp * (dn.x + dp.x);
+            if (ten != 0.f) {  // Eq. membraneforce
+                const float ln = sqrtf(dn.x * dn.x + dn.y * dn.y);
+                const float lp = sqrtf(dp.x * dp.x + dp.y * dp.y);
+                Fx += ten * (dn.x / ln - dp.x / lp);
+                Fy += ten * (dn.y / ln - dp.y / lp);
+            }
+            if (OPTS && a.jpartner) {  // Eq. celljunctionforce (a launch without the move)
+                const float2 J = junction_force32(a, sx[t], a.jpartner[v0 + t]);
+                Fx += J.x;
+                Fy += J.y;
+            }
+            if (a.write_vforce) a.vforce[v0 + t] = make_double2((double)Fx, (double)Fy);
+
+            float wx[4], wy[4];
+            weights_from_frac(f.x, wx);
+            weights_from_frac(f.y, wy);
+            const int x0 = wrap_near(b.x - 1, a.nx);
+            const bool seam = x0 + 3 >= a.nx, odd = x0 & 1;
+            int J = a.bc_y ? b.y - 1 : wrap_near(b.y - 1, a.ny);
+            uint8_t* mark = S.grp + (b.y - 1 - gb.row0) * kGroupCols + ((x0 >> 2) - gb.g0);
+            const int mark2 = ((x0 + 3) >> 2) - (x0 >> 2);
+#pragma unroll
+            for (int j = 0; j < 4; ++j, ++J) {
+                if (a.bc_y) {
+                    if (J < 0 || J >= a.ny) {
+                        raise_flag(a.diag, kDiagWallStencil);
+                        continue;
+                    }
+                } else if (J >= a.ny) {
+                    J -= a.ny;
+                }
+                float2* row = force + J * pitch;
+                float cx4[4], cy4[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const float w = wx[i] * wy[j];
+                    cx4[i] = Fx * w;
+                    cy4[i] = Fy * w;
+                }
+                // the four nodes of the row: two aligned 16-byte reductions
+                // when it starts on an even node, 8 + 16 + 8 bytes when it
+                // starts on an odd one, one per node across the periodic seam
+                if (!seam) {
+                    float2* r0 = row + x0;
+                    if (!odd) {
+                        force_red2(a, r0, cx4[0], cy4[0], cx4[1], cy4[1]);
+                        force_red2(a, r0 + 2, cx4[2], cy4[2], cx4[3], cy4[3]);
+                    } else {
+                        force_red1(a, r0, cx4[0], cy4[0]);
+                        force_red2(a, r0 + 1, cx4[1], cy4[1], cx4[2], cy4[2]);
+                        force_red1(a, r0 + 3, cx4[3], cy4[3]);
+                    }
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+                        spread_add(a, row + (x0 + i >= a.nx ? x0 + i - a.nx : x0 + i), cx4[i],
+                                   cy4[i]);
+                }
+                if (GROUPS && gb.fits) {
+                    mark[j * kGroupCols] = 1;
+                    mark[j * kGroupCols + mark2] = 1;
+                } else {
+                    int ix[4];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) ix[i] = x0 + i >= a.nx ? x0 + i - a.nx : x0 + i;
+                    mark_row(a, a.fmask, (int64_t)J * pitch, ix);
+                }
+            }
         }
     }
-    if (!labels) return;  // uniform over the CTA
-    cell_sync<NT>(bar);
-    if (INLINE_FILL)
-        fill_labels_body(a, c, n, sx, rowcnt, thr, scan && s_flag == 0, I0, J0, rows, cols, tid,
-                         NT);
-    else
-        fill_labels_call(a, c, n, sx, rowcnt, thr, scan && s_flag == 0, I0, J0, rows, cols, tid,
-                         NT);
+    // the label fill needs the crossings only (complete since the barrier)
+    if (labels) {
+        if (INLINE_FILL)
+            fill_labels_body(a, c, n, sx, rowcnt, thr, scan && s_flag == 0, I0, J0, rows, cols,
+                             tid, NT);
+        else
+            fill_labels_call(a, c, n, sx, rowcnt, thr, scan && s_flag == 0, I0, J0, rows, cols,
+                             tid, NT);
+    }
+    if (GROUPS && gb.fits) {  // uniform over the CTA
+        cell_sync<NT>(bar);
+        flush_groups<NT>(a, gb, S.grp, tid);
+    }
 }
 
 }  // namespace lbib

@@ -331,58 +331,43 @@ __device__ __forceinline__ double min_image(double d, int n) {
 // shared memory of the FP32 per-cell IB work (one CTA per cell), as pointers
 // into the CTA's shared memory; the vertex arrays hold `maxv` entries
 struct IBShared32 {
-    double2* sx;  // FP64 positions (exact fallbacks)
-    int2* sb;     // floor(X)
-    float2* sf;   // X - floor(X)
-    int* rowcnt;  // kMaxRows
-    int* thr;     // kMaxRows * kMaxCross
-    int* sbox;    // 4
-    int* s_flag;  // 1
-    // the cell's force-mask words (kMaskTable keys and bits): the spreading
-    // ORs its group bits here and the CTA then ORs each distinct word into
-    // the mask once
-    uint32_t* mkey;
-    uint32_t* mval;
+    double2* sx;   // FP64 positions (exact fallbacks)
+    int2* sb;      // floor(X)
+    float2* sf;    // X - floor(X)
+    float* spr;    // spring force of the edge to the next vertex, over the edge vector
+    uint8_t* grp;  // kGroupRows x kGroupCols: the 4-node groups that receive force
+    int4* wbox;    // each warp's bounding box (at most 8 warps)
+    int* rowcnt;   // kMaxRows
+    int* thr;      // kMaxRows * kMaxCross
+    int* s_flag;   // 1
     int maxv;
 };
 
-constexpr int kMaskTableLog2 = 8;
-constexpr int kMaskTable = 1 << kMaskTableLog2;
-constexpr uint32_t kMaskEmpty = 0xFFFFFFFFu;
+// the table of a cell's force groups: 16 groups (64 nodes) wide, one 16-byte
+// row per lattice row
+constexpr int kGroupCols = 16, kGroupRows = 128;
 
 // fixed part of the FP32 IB kernel's dynamic shared memory (bytes, 16-aligned)
 constexpr int kIBSmemFixed =
-    ((kMaxRows + kMaxRows * kMaxCross + 4 + 1 + 2 * kMaskTable) * 4 + 15) / 16 * 16;
-constexpr int kIBSmemPerVertex = 16 + 8 + 8;
+    kGroupRows * kGroupCols + 8 * 16 + ((kMaxRows + kMaxRows * kMaxCross + 1) * 4 + 15) / 16 * 16;
+constexpr int kIBSmemPerVertex = 16 + 8 + 8 + 4;
 
 // the views of one cell slot of that shared memory (fixed part, then maxv
-// vertices)
+// vertices, maxv a multiple of 8)
 __device__ __forceinline__ IBShared32 ib_shared32_view(unsigned char* base, int maxv) {
     IBShared32 v;
-    int* fixed = reinterpret_cast<int*>(base);
-    v.rowcnt = fixed;
-    v.thr = fixed + kMaxRows;
-    v.sbox = v.thr + kMaxRows * kMaxCross;
-    v.s_flag = v.sbox + 4;
-    v.mkey = reinterpret_cast<uint32_t*>(v.s_flag + 1);
-    v.mval = v.mkey + kMaskTable;
+    v.grp = base;
+    v.wbox = reinterpret_cast<int4*>(base + kGroupRows * kGroupCols);
+    v.rowcnt = reinterpret_cast<int*>(v.wbox + 8);
+    v.thr = v.rowcnt + kMaxRows;
+    v.s_flag = v.thr + kMaxRows * kMaxCross;
     v.sx = reinterpret_cast<double2*>(base + kIBSmemFixed);
     v.sb = reinterpret_cast<int2*>(v.sx + maxv);
     v.sf = reinterpret_cast<float2*>(v.sb + maxv);
+    v.spr = reinterpret_cast<float*>(v.sf + maxv);
     v.maxv = maxv;
     return v;
 }
-
-// a static shared-memory block for the largest cells (the persistent kernel)
-struct IBSmem32 {
-    double2 sx[kMaxVertsPerCell];  // FP64 positions (exact fallbacks)
-    int2 sb[kMaxVertsPerCell];     // floor(X)
-    float2 sf[kMaxVertsPerCell];   // X - floor(X)
-    int rowcnt[kMaxRows];
-    int thr[kMaxRows * kMaxCross];
-    int sbox[4];
-    int s_flag;
-};
 
 // Programmatic dependent launch.  A kernel launched with the programmatic
 // stream-serialization attribute may start while the previous kernel of its
