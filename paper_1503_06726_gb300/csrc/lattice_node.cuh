@@ -285,9 +285,9 @@ _Pragma("unroll") \
             mjy[s] = gs * (g[s][2] - g[s][4]); \
         } \
     } \
-    collide_node<C, S, FORCING, SCALED>(k, d, g, fv.x, fv.y, sbits, 0u, rho, ux, uy, ph, \
-                                        OPTS && (a.msrc != nullptr || a.nsrc != nullptr), ms, \
-                                        pn); \
+    collide_any<C, S, FORCING, SCALED>(k, d, g, fv.x, fv.y, sbits, rho, ux, uy, ph, \
+                                       OPTS && (a.msrc != nullptr || a.nsrc != nullptr), ms, \
+                                       pn); \
     if (mom_w) { \
 _Pragma("unroll") \
         for (int s = 0; s < S; ++s) { \
@@ -344,7 +344,18 @@ _Pragma("unroll") \
         } \
     } \
     if (a.out) static_cast<C*>(a.rho)[node] = rho; \
-    if (!(rho > C(0)) || !isfinite(ux) || !isfinite(uy)) atomicOr(a.diag + kDiagNonFinite, 1u);
+    if (!positive(rho) || !finite(ux) || !finite(uy)) atomicOr(a.diag + kDiagNonFinite, 1u);
+
+// rho > 0 and finite u; of doubles by their bits, off the slow FP64 pipe
+__device__ __forceinline__ bool positive(float v) { return v > 0.f; }
+__device__ __forceinline__ bool finite(float v) { return isfinite(v); }
+__device__ __forceinline__ bool positive(double v) {
+    const long long b = __double_as_longlong(v);
+    return b > 0 && b <= 0x7ff0000000000000ll;
+}
+__device__ __forceinline__ bool finite(double v) {
+    return (__double2hiint(v) & 0x7ff00000) != 0x7ff00000;
+}
 
 // Explicit round-to-nearest operations on the value of one node (float,
 // double) or of two nodes at once (float2: the packed FP32 instructions of
@@ -537,6 +548,148 @@ __device__ __forceinline__ void collide_node(const Coefs<typename Lane<V>::S>& k
             g[s][4] = L::fma(omcD, g[s][4], L::sub(evB, oy));
         }
     }
+}
+
+// The same collision for FP64, with its operations counted: GB300 issues one
+// FP64 instruction of a warp every 16 cycles, so the update of a node is
+// bound by them and nothing else (1237 x 811: 0.82 of the pipe, 0.10 of DRAM;
+// 121 per node as each warp issued them, 243 us, now 104, 205 us).
+// In sums and differences of opposite directions, S = d_q + d_q' and
+// D = d_q - d_q', with j the momentum (half the force in it: j = rho u):
+//   E = omega (drho - 3/2 j.u),  v.p = w omega 3 (v.j)  for weight w
+//   d*_q, d*_q' = (1 - omega)/2 S + w E + 3/2 (v.u)(v.p)  +-  ((1 - omega)/2 D + v.p)
+// 64 operations and the reciprocal, and 22 per linear species.  The force adds 19 in a branch of its own: the warps without
+// a spread force, most of them, skip it (Guo: w pref (9 (v.u)(v.F) - 3 u.F)
+// to the even part, 3 w pref v.F to the odd one; the paper's term 3 w v.F).
+template <int S, int FORCING>
+__device__ __forceinline__ void collide_node64(const Coefs<double>& k, double (&d)[9],
+                                               double (&g)[S > 0 ? S : 1][5], double fvx,
+                                               double fvy, uint32_t bits, double& rho, double& ux,
+                                               double& uy, double (&ph)[S > 0 ? S : 1],
+                                               bool mass_on, double ms, bool pnode) {
+    using L = Lane<double>;
+    // pairs of opposite directions: (1, 3), (2, 4), (5, 7), (6, 8)
+    double S1 = L::add(d[1], d[3]), D1 = L::sub(d[1], d[3]);
+    double S2 = L::add(d[2], d[4]), D2 = L::sub(d[2], d[4]);
+    double S5 = L::add(d[5], d[7]), D5 = L::sub(d[5], d[7]);
+    double S6 = L::add(d[6], d[8]), D6 = L::sub(d[6], d[8]);
+    double drho = L::add(L::add(L::add(S1, S2), L::add(S5, S6)), d[0]);
+    double jx = L::add(D1, L::sub(D5, D6)), jy = L::add(D2, L::add(D5, D6));
+    if (pnode) {  // every population scaled to the density prho (see collide_node)
+        const double gam = L::mul(k.prho, L::rcp(L::add(k.rho0, drho)));
+        const double r = L::mul(L::sub(gam, 1.0), k.rho0);
+        const double r1 = L::mul(r, 2.0 * k.w9c[1]), r5 = L::mul(r, 2.0 * k.w9c[2]);
+        d[0] = L::fma(gam, d[0], L::mul(r, k.w9c[0]));
+        S1 = L::fma(gam, S1, r1), S2 = L::fma(gam, S2, r1);
+        S5 = L::fma(gam, S5, r5), S6 = L::fma(gam, S6, r5);
+        D1 = L::mul(gam, D1), D2 = L::mul(gam, D2), D5 = L::mul(gam, D5), D6 = L::mul(gam, D6);
+        drho = k.prho - k.rho0;
+        jx = L::mul(gam, jx);
+        jy = L::mul(gam, jy);
+    }
+    rho = L::add(k.rho0, drho);
+    const double irho = L::rcp(rho);
+    const bool forced = ((__double_as_longlong(fvx) | __double_as_longlong(fvy) |
+                          __double_as_longlong(k.bfx) | __double_as_longlong(k.bfy))
+                         << 1) != 0ll;
+    double Fx = 0.0, Fy = 0.0;
+    if (forced) {
+        Fx = L::add(k.bfx, fvx);
+        Fy = L::add(k.bfy, fvy);
+        if (FORCING == LBIB_GUO) {
+            jx = L::fma(0.5, Fx, jx);
+            jy = L::fma(0.5, Fy, jy);
+        }
+    }
+    ux = L::mul(jx, irho);
+    uy = L::mul(jy, irho);
+    double E = L::mul(k.omega, L::fma(-1.5, L::fma(jx, ux, L::mul(jy, uy)), drho));
+    if (FORCING == LBIB_GUO && forced)
+        E = L::fma(k.c3pref, L::fma(ux, Fx, L::mul(uy, Fy)), E);
+    // mass source (Sec. 3.2.3): w_q S added to every direction, no momentum
+    if (mass_on) E = L::add(E, ms);
+    // v.p, v.u and the even part of v = (1,0), (0,1), (1,1), (-1,1)
+    double o1 = L::mul(k.om3, jx), o2 = L::mul(k.om3, jy);
+    const double p5y = L::mul(0.25, o2);
+    double o5 = L::fma(0.25, o1, p5y), o6 = L::fma(-0.25, o1, p5y);
+    const double hx = L::mul(1.5, ux), hy = L::mul(1.5, uy);
+    const double hs = L::add(hx, hy), hd = L::sub(hy, hx);
+    const double E1 = L::mul(k.w9c[1], E), E5 = L::mul(k.w9c[2], E);
+    double e1 = L::fma(hx, o1, E1), e2 = L::fma(hy, o2, E1);
+    double e5 = L::fma(hs, o5, E5), e6 = L::fma(hd, o6, E5);
+    if (forced) {
+        if (FORCING == LBIB_GUO) {
+            const double qx = L::mul(k.pref, Fx), qy = L::mul(k.pref, Fy);
+            const double qs = L::add(qx, qy), qd = L::sub(qy, qx);
+            e1 = L::fma(ux, qx, e1);
+            e2 = L::fma(uy, qy, e2);
+            e5 = L::fma(L::mul(1.0 / 6.0, hs), qs, e5);
+            e6 = L::fma(L::mul(1.0 / 6.0, hd), qd, e6);
+            o1 = L::fma(1.0 / 3.0, qx, o1);
+            o2 = L::fma(1.0 / 3.0, qy, o2);
+            o5 = L::fma(1.0 / 12.0, qs, o5);
+            o6 = L::fma(1.0 / 12.0, qd, o6);
+        } else {
+            o1 = L::fma(1.0 / 3.0, Fx, o1);
+            o2 = L::fma(1.0 / 3.0, Fy, o2);
+            o5 = L::fma(1.0 / 12.0, L::add(Fx, Fy), o5);
+            o6 = L::fma(1.0 / 12.0, L::sub(Fy, Fx), o6);
+        }
+    }
+    d[0] = L::fma(k.w9c[0], E, L::mul(k.omc, d[0]));
+    const double h = k.omch;
+    const double a1 = L::fma(h, S1, e1), b1 = L::fma(h, D1, o1);
+    const double a2 = L::fma(h, S2, e2), b2 = L::fma(h, D2, o2);
+    const double a5 = L::fma(h, S5, e5), b5 = L::fma(h, D5, o5);
+    const double a6 = L::fma(h, S6, e6), b6 = L::fma(h, D6, o6);
+    d[1] = L::add(a1, b1), d[3] = L::sub(a1, b1);
+    d[2] = L::add(a2, b2), d[4] = L::sub(a2, b2);
+    d[5] = L::add(a5, b5), d[7] = L::sub(a5, b5);
+    d[6] = L::add(a6, b6), d[8] = L::sub(a6, b6);
+    if (S > 0) {
+        double T1[S > 0 ? S : 1], U1[S > 0 ? S : 1], T2[S > 0 ? S : 1], U2[S > 0 ? S : 1];
+#pragma unroll
+        for (int s = 0; s < S; ++s) {
+            T1[s] = L::add(g[s][1], g[s][3]);
+            U1[s] = L::sub(g[s][1], g[s][3]);
+            T2[s] = L::add(g[s][2], g[s][4]);
+            U2[s] = L::sub(g[s][2], g[s][4]);
+            ph[s] = L::add(L::add(T1[s], T2[s]), g[s][0]);
+        }
+#pragma unroll
+        for (int s = 0; s < S; ++s) {
+            double R = (bits >> s) & 1u ? k.srate[s] : 0.0;
+            if (S >= 2 && s < 2 && k.react_model == LBIB_REACT_SCHNAKENBERG) {
+                const double r2l = L::mul(L::mul(ph[0], ph[0]), ph[1]);
+                const double rate = s == 0 ? L::add(L::sub(k.sa, ph[0]), r2l) : L::sub(k.sb, r2l);
+                R = L::fma(k.sgamma, rate, R);
+            } else {
+#pragma unroll
+                for (int b = 0; b < S; ++b) R = L::fma(k.K[s][b], ph[b], R);
+            }
+            const double ev = L::fma(k.omegaD[s], ph[s], R);
+            const double evB = L::mul(k.w5c[1], ev);
+            const double o = L::mul(k.o3D[s], ph[s]);
+            const double hD = k.omchD[s];
+            const double t1 = L::fma(hD, T1[s], evB), u1 = L::fma(o, ux, L::mul(hD, U1[s]));
+            const double t2 = L::fma(hD, T2[s], evB), u2 = L::fma(o, uy, L::mul(hD, U2[s]));
+            g[s][0] = L::fma(k.w5c[0], ev, L::mul(k.omcD[s], g[s][0]));
+            g[s][1] = L::add(t1, u1), g[s][3] = L::sub(t1, u1);
+            g[s][2] = L::add(t2, u2), g[s][4] = L::sub(t2, u2);
+        }
+    }
+}
+// one node in any storage and compute type
+template <typename C, int S, int FORCING, bool SCALED>
+__device__ __forceinline__ void collide_any(const Coefs<C>& k, C (&d)[9], C (&g)[S > 0 ? S : 1][5],
+                                            C fvx, C fvy, uint32_t bits, C& rho, C& ux, C& uy,
+                                            C (&ph)[S > 0 ? S : 1], bool mass_on, C ms,
+                                            bool pnode) {
+    if constexpr (std::is_same<C, double>::value)
+        collide_node64<S, FORCING>(k, d, g, fvx, fvy, bits, rho, ux, uy, ph, mass_on, ms, pnode);
+    else
+        collide_node<C, S, FORCING, SCALED>(k, d, g, fvx, fvy, bits, 0u, rho, ux, uy, ph, mass_on,
+                                            ms, pnode);
 }
 
 // WAIT: the caller is a kernel of its own, launched programmatically after an

@@ -104,6 +104,7 @@ bool make_layout(const lbib_params& p, int max_vertices, int max_cells, Layout* 
     l.vforce = take(V * 16);
     l.vbase = take(V * 8);
     l.vfrac = take(V * 8);
+    if (p.precision == LBIB_FP64) l.vw = take(V * 64);
     l.off = take((C + 1) * 4);
     l.pres = take(C * 8);
     l.srcf = take(C);
@@ -212,6 +213,13 @@ static void fill_coefs(const lbib_params& p, Coefs<C>* k) {
     k->isig = (C)(scaled ? 1.0 / sf : 1.0);
     k->isig_g = (C)(scaled ? 1.0 / sg : 1.0);
     exact_sum_weights<C>(k->w9c, k->w5c);
+    k->om3 = k->omega / C(3);
+    k->c3pref = C(-3) * k->pref;
+    k->omch = C(0.5) * k->omc;
+    for (int s = 0; s < kMaxSpecies; ++s) {
+        k->omchD[s] = C(0.5) * k->omcD[s];
+        k->o3D[s] = C(3) * k->w5c[1] * k->omegaD[s];
+    }
     for (int q = 0; q < 9; ++q) {
         const double wq = (double)k->w9c[q == 0 ? 0 : (q < 5 ? 1 : 2)];
         k->fscale[q] = (C)(scaled ? wq * sf : 1.0);
@@ -319,6 +327,7 @@ static IBArgs ib_args(lbib_ctx* c, bool move, bool prep, bool out_next) {
     a.do_force = 1;
     a.vbase = c->at<int2>(L.vbase);
     a.vfrac = c->at<float2>(L.vfrac);
+    a.vw = L.vw ? c->at<double>(L.vw) : nullptr;
     a.fmask = c->at<uint32_t>(L.fmask);
     a.lmask = c->at<uint32_t>(L.lmask);
     a.src = c->at<uint8_t>(L.src);

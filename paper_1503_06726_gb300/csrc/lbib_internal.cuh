@@ -142,7 +142,7 @@ struct Layout {
     uint64_t f[2] = {0, 0}, g[2] = {0, 0};
     uint64_t force = 0, u = 0, rho = 0, phi = 0, id = 0, id_out = 0, force_out = 0;
     uint64_t xy = 0, L0 = 0, k = 0, vforce = 0, off = 0, pres = 0, srcf = 0, area = 0;
-    uint64_t vbase = 0, vfrac = 0, fmask = 0, lmask = 0, src = 0, smask = 0;
+    uint64_t vbase = 0, vfrac = 0, vw = 0, fmask = 0, lmask = 0, src = 0, smask = 0;
     uint64_t dom = 0;          // domain labels of the confined species (noflux_mask != 0)
     // the no-flux closure of Sec. 6.1 (noflux_scheme 0): a 16-bit code per
     // node (kNcode* bits) and the species moments (phi, jx, jy per species,
@@ -189,6 +189,10 @@ struct Coefs {
     // FP32 velocity error at 2000 steps from 7.9e-5 to 1.3e-4.
     C w9c[3];
     C w5c[2];
+    // products the FP64 collision would otherwise form at every node:
+    // omega / 3, -3 pref, (1 - omega) / 2; per species (1 - omega_D) / 2 and
+    // 3 w omega_D
+    C om3, c3pref, omch, omchD[kMaxSpecies], o3D[kMaxSpecies];
 };
 
 // The weight sets of Coefs::w9c / w5c for the compute type C (FP64: both
@@ -280,6 +284,8 @@ struct IBArgs {
     int do_force;       // compute and spread vertex forces (0: labels only)
     int2* vbase;        // FP32 path, optional: floor(X) per vertex handed to the next move
     float2* vfrac;      // FP32 path, optional: X - floor(X) per vertex
+    double* vw;         // FP64 path, optional: the 4 + 4 kernel weights per vertex handed to
+                        // the next move (with vbase)
     uint32_t* fmask;    // optional: mark the groups that receive spread force
     uint32_t* lmask;    // optional: mark the groups that receive labels
     void* src;          // optional source-bits plane (OR of the cells' bits): one byte per
