@@ -113,6 +113,11 @@ __global__ void __launch_bounds__(kLatticeThreads, PairOccupancy<S>::kMinBlocks)
          !LBIB_CHK_INDEX(a.diag, kSiteMask, (int64_t)(node >> 7), mask_words(a.plane))))
         valid = false;
 
+    // without cells the launch before wrote them: wait for it first
+    if (!a.ib) {
+        griddep_wait();
+        griddep_launch_dependents();
+    }
     // ---- every population word first (written two launches back: L2 path)
     const uint64_t pol = a.l2_first ? l2_evict_first() : l2_evict_normal();
     const uint32_t* F = static_cast<const uint32_t*>(a.fsrc);
@@ -501,6 +506,11 @@ __global__ void __launch_bounds__(kLatticeThreads, QuadOccupancy<S>::kMinBlocks)
          !LBIB_CHK_INDEX(a.diag, kSiteMask, (int64_t)(node >> 7), mask_words(a.plane))))
         valid = false;
 
+    // without cells the launch before wrote them: wait for it first
+    if (!a.ib) {
+        griddep_wait();
+        griddep_launch_dependents();
+    }
     // ---- every population word first (written two launches back: L2 path)
     const uint64_t pol = a.l2_first ? l2_evict_first() : l2_evict_normal();
     const uint2* F = static_cast<const uint2*>(a.fsrc);

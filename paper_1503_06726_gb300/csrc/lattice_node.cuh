@@ -95,42 +95,36 @@ __device__ __forceinline__ void pull5_closure(const T* B, int64_t P, const C* M,
                                               int x, int xm, int xp, int xmm, int xpp, bool lo,
                                               bool hi, uint64_t pol, C isg, C wq, C g[5],
                                               uint32_t* diag) {
-    using St = Store<T, C>;
-    g[0] = St::ld(B + node, pol);
+    // every population as if none were missing: these loads wait for nothing,
+    // not even for the node's code (with the missing ones skipped, the loads
+    // came a round trip after it)
+    pull5<T, C, WALLS>(B, P, node, r0, rm, rp, x, xm, xp, lo, hi, pol, g);
+    if (((code >> kNcodeMiss) & 0xFu) == 0u) return;
+    // then the missing ones, all their moments loaded before any is used
+    C p1[5], j1[5], p2[5];
 #pragma unroll
     for (int q = 1; q <= 4; ++q) {
+        p1[q] = j1[q] = p2[q] = C(0);
         if ((code >> (kNcodeMiss + q - 1)) & 1u) {
             const int i1 = q == 1 ? r0 + xp : (q == 3 ? r0 + xm : (q == 2 ? rp + x : rm + x));
             const int i2 = q == 1 ? r0 + xpp : (q == 3 ? r0 + xmm : (q == 2 ? rpp + x : rmm + x));
             if (!LBIB_CHK_INDEX(diag, kSiteClosureIndex, i1, P) ||
-                !LBIB_CHK_INDEX(diag, kSiteClosureIndex, i2, P)) {
-                g[q] = C(0);
+                !LBIB_CHK_INDEX(diag, kSiteClosureIndex, i2, P))
                 continue;
-            }
             const bool in1 = (code >> (kNcodeIn1 + q - 1)) & 1u;
             const bool in2 = (code >> (kNcodeIn2 + q - 1)) & 1u;
-            const C* Mj = M + (q == 1 || q == 3 ? P : 2 * P);
-            C ph, jc;
-            if (in1) {
-                const C p1 = __ldcg(M + i1);
-                const C j1 = __ldcg(Mj + i1);
-                ph = in2 ? C(2) * p1 - __ldcg(M + i2) : p1;
-                jc = (q == 1 || q == 2) ? j1 : -j1;
-            } else {
-                ph = __ldcg(M + node);
-                jc = C(0);
-            }
+            p1[q] = __ldcg(M + (in1 ? i1 : node));
+            if (in1) j1[q] = __ldcg(M + (q == 1 || q == 3 ? P : 2 * P) + i1);
+            if (in2) p2[q] = __ldcg(M + i2);
+        }
+    }
+#pragma unroll
+    for (int q = 1; q <= 4; ++q) {
+        if ((code >> (kNcodeMiss + q - 1)) & 1u) {
+            const bool in2 = (code >> (kNcodeIn2 + q - 1)) & 1u;
+            const C ph = in2 ? C(2) * p1[q] - p2[q] : p1[q];
+            const C jc = (q == 1 || q == 2) ? j1[q] : -j1[q];
             g[q] = SCALED ? (ph + jc) * isg : wq * (ph + jc);
-        } else if (q == 1) {
-            g[1] = St::ld((B + 1 * P) + (r0 + xm), pol);
-        } else if (q == 3) {
-            g[3] = St::ld((B + 3 * P) + (r0 + xp), pol);
-        } else if (q == 2) {
-            g[2] = (WALLS && lo) ? St::ld((B + 4 * P) + node, pol)
-                                 : St::ld((B + 2 * P) + (rm + x), pol);
-        } else {
-            g[4] = (WALLS && hi) ? St::ld((B + 2 * P) + node, pol)
-                                 : St::ld((B + 4 * P) + (rp + x), pol);
         }
     }
 }
@@ -179,6 +173,12 @@ __device__ __forceinline__ void pull5_closure(const T* B, int64_t P, const C* M,
         !LBIB_CHK_INDEX(a.diag, kSiteMask, (int64_t)(node >> 7), mask_words(a.plane))) \
         return; \
  \
+    /* without cells the launch before is the lattice update whose populations */ \
+    /* this one reads: wait for it first */ \
+    if (GRIDDEP && !a.ib) { \
+        griddep_wait(); \
+        griddep_launch_dependents(); \
+    } \
     /* ---- every load of the node first (all independent, read-only path), so */ \
     /* that a thread has all its DRAM requests in flight at once */ \
     const T* F = static_cast<const T*>(a.fsrc); \
@@ -558,9 +558,10 @@ __device__ __forceinline__ void collide_node(const Coefs<typename Lane<V>::S>& k
 // D = d_q - d_q', with j the momentum (half the force in it: j = rho u):
 //   E = omega (drho - 3/2 j.u),  v.p = w omega 3 (v.j)  for weight w
 //   d*_q, d*_q' = (1 - omega)/2 S + w E + 3/2 (v.u)(v.p)  +-  ((1 - omega)/2 D + v.p)
-// 64 operations and the reciprocal, and 22 per linear species.  The force adds 19 in a branch of its own: the warps without
-// a spread force, most of them, skip it (Guo: w pref (9 (v.u)(v.F) - 3 u.F)
-// to the even part, 3 w pref v.F to the odd one; the paper's term 3 w v.F).
+// 64 operations and the reciprocal, and 22 per linear species.  The force adds
+// 19 in a branch of its own: the warps without a spread force, most of them,
+// skip it (Guo: w pref (9 (v.u)(v.F) - 3 u.F) to the even part, 3 w pref v.F to
+// the odd one; the paper's term 3 w v.F).
 template <int S, int FORCING>
 __device__ __forceinline__ void collide_node64(const Coefs<double>& k, double (&d)[9],
                                                double (&g)[S > 0 ? S : 1][5], double fvx,

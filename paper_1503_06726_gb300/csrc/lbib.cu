@@ -354,7 +354,8 @@ IBArgs ctx_ib_args(lbib_ctx* c, bool move, bool prep, bool out_next) {
 // pdl: programmatic launch, allowed only when the previous launch on the
 // stream is the other kernel of the step (an IB launch before a lattice
 // launch and vice versa): each kernel's early loads rely on the launch two
-// back having completed, which the other kernel's wait guarantees.
+// back having completed, which the other kernel's wait guarantees.  Without
+// cells lattice launches follow one another and wait before any load.
 // The no-flux closure reads the species moments of the previous step; after
 // create, lbib_set_species, lbib_set_domains or lbib_set_state there is no
 // previous step, and the moments of the stored populations stand in.
@@ -371,7 +372,7 @@ static cudaError_t enqueue_lattice(lbib_ctx* c, int src_buf, bool out, bool pdl 
     NvtxRange nvtx_range("lbib.lattice_update");
     LatticeArgs a = lattice_args(c, src_buf, out);
     return launch_lattice(c->p.precision, c->p.n_species, c->p.bc_y, c->p.forcing, a,
-                          coefs_of(c), c->block, c->stream, pdl && c->nC > 0, c->lattice_npt);
+                          coefs_of(c), c->block, c->stream, pdl, c->lattice_npt);
 }
 
 static cudaError_t enqueue_ib(lbib_ctx* c, bool move, bool prep, bool out_next,
@@ -876,7 +877,7 @@ int lbib_step(lbib_ctx* c, int32_t n_steps) {
         const bool last = (left == 1);
         e = enqueue_lattice(c, c->cur, last, follows_kernel);
         if (e == cudaSuccess && ib) e = enqueue_ib(c, true, !last, left == 2, true);
-        follows_kernel = ib;
+        follows_kernel = true;
         c->cur = 1 - c->cur;
         --left;
     }
