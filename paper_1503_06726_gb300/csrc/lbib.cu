@@ -393,26 +393,40 @@ static void drop_graphs(lbib_ctx* c) {
             cudaGraphExecDestroy(c->tail[i]);
             c->tail[i] = nullptr;
         }
+        if (c->lchunk[i]) {
+            cudaGraphExecDestroy(c->lchunk[i]);
+            c->lchunk[i] = nullptr;
+        }
     }
     c->chunk_nC = -1;
 }
 
-// two full steps starting from buffer parity `par`, ending with the prep of
-// the following step: [lat(par), ib move+prep, lat(1-par), ib move+prep];
-// inside the graph each launch after the first is programmatic
-// tail: the second IB launch only moves (no prep for a following step)
-static cudaError_t enqueue_chunk(lbib_ctx* c, int par, bool tail = false) {
-    cudaError_t e = enqueue_lattice(c, par, false);
-    if (e == cudaSuccess) e = enqueue_ib(c, true, true, false, true);
-    if (e == cudaSuccess) e = enqueue_lattice(c, 1 - par, false, true);
-    if (e == cudaSuccess) e = enqueue_ib(c, true, !tail, false, true);
+// `pairs` times two full steps starting from buffer parity `par`, ending with
+// the prep of the following step: [lat(par), ib move+prep, lat(1-par), ib
+// move+prep]; inside the graph each launch after the first is programmatic
+// tail: the last IB launch only moves (no prep for a following step)
+static cudaError_t enqueue_chunk(lbib_ctx* c, int par, int pairs, bool tail = false) {
+    cudaError_t e = cudaSuccess;
+    for (int i = 0; i < pairs && e == cudaSuccess; ++i) {
+        e = enqueue_lattice(c, par, false, i > 0);
+        if (e == cudaSuccess) e = enqueue_ib(c, true, true, false, true);
+        if (e == cudaSuccess) e = enqueue_lattice(c, 1 - par, false, true);
+        if (e == cudaSuccess) e = enqueue_ib(c, true, !(tail && i == pairs - 1), false, true);
+    }
     return e;
 }
 
-static cudaError_t get_chunk_graph(lbib_ctx* c, int par, cudaGraphExec_t* out,
+// A graph's launch leaves the device idle for about a microsecond before it,
+// so a context that has been asked for many steps replays eight pairs at a
+// time (1024^2, 400 cells: 36.2 -> 34.2 us per step).  The long graph takes about 0.4 ms to build, 10 us for each
+// of its nodes, which is why the first kLongAfter steps do without.
+constexpr int kLongChunk = 8;
+constexpr int64_t kLongAfter = 512;
+
+static cudaError_t get_chunk_graph(lbib_ctx* c, int par, cudaGraphExec_t* out, int pairs,
                                    bool tail = false) {
     if (c->chunk_nC != c->nC) drop_graphs(c);
-    cudaGraphExec_t* slot = tail ? &c->tail[par] : &c->chunk[par];
+    cudaGraphExec_t* slot = tail ? &c->tail[par] : (pairs > 1 ? &c->lchunk[par] : &c->chunk[par]);
     if (!*slot) {
         cudaStream_t cap;
         cudaError_t e = cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking);
@@ -422,7 +436,7 @@ static cudaError_t get_chunk_graph(lbib_ctx* c, int par, cudaGraphExec_t* out,
         cudaGraph_t g = nullptr;
         e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
         if (e == cudaSuccess) {
-            cudaError_t e2 = enqueue_chunk(c, par, tail);
+            cudaError_t e2 = enqueue_chunk(c, par, pairs, tail);
             e = cudaStreamEndCapture(cap, &g);
             if (e2 != cudaSuccess) e = e2;
         }
@@ -863,12 +877,15 @@ int lbib_step(lbib_ctx* c, int32_t n_steps) {
     // full two-step chunks through the graph, keeping the last two steps apart
     // (they write the vertex forces and the output fields)
     bool graphed = false;
+    c->steps_asked += n_steps;
     while (e == cudaSuccess && left > 3) {
         cudaGraphExec_t g;
-        e = get_chunk_graph(c, c->cur, &g);
+        const int pairs =
+            c->steps_asked >= kLongAfter && left >= 2 * kLongChunk + 2 ? kLongChunk : 1;
+        e = get_chunk_graph(c, c->cur, &g, pairs);
         if (e == cudaSuccess) e = cudaGraphLaunch(g, c->stream);
         graphed = true;
-        left -= 2;
+        left -= 2 * pairs;
     }
     // the remaining steps as single launches: a launch that directly follows
     // the other kernel of the step (not a graph) is programmatic
@@ -914,11 +931,14 @@ int lbib_advance(lbib_ctx* c, int32_t n_steps) {
         --left;
     }
     if (e == cudaSuccess && left > 0) e = rb_fence(c, c->stream);
+    c->steps_asked += n_steps;
     while (e == cudaSuccess && left > 0) {
         cudaGraphExec_t g;
-        e = get_chunk_graph(c, c->cur, &g, left == 2);
+        const int pairs =
+            c->steps_asked >= kLongAfter && left >= 2 * kLongChunk + 2 ? kLongChunk : 1;
+        e = get_chunk_graph(c, c->cur, &g, pairs, left == 2);
         if (e == cudaSuccess) e = cudaGraphLaunch(g, c->stream);
-        left -= 2;
+        left -= 2 * pairs;
     }
     if (e != cudaSuccess) return cuda_fail(c, e, "lbib_advance");
     // the lattice fields, labels and vertex forces of the last step were not written

@@ -32,6 +32,9 @@ struct lbib_ctx {
     // the same two steps whose last IB launch only moves (the end of an
     // lbib_advance call), keyed the same way
     cudaGraphExec_t tail[2] = {nullptr, nullptr};
+    // kLongChunk such pairs in one graph, for contexts that run many steps
+    cudaGraphExec_t lchunk[2] = {nullptr, nullptr};
+    int64_t steps_asked = 0;  // steps of lbib_step / lbib_advance since create
     int chunk_nC = -1;
     // pinned staging of lbib_set_cell_params (pressure then source flags), and
     // the event of its last upload (the buffer is reused once that is done)
