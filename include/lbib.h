@@ -405,11 +405,14 @@ int lbib_steady_solve(int32_t nx, int32_t ny, int32_t batch, const uint8_t* d_sr
  * size, tau, boundary -- and its own cells) in one caller-owned workspace and
  * advances all of them by one persistent cooperative kernel launch per
  * lbib_ensemble_step() call (LBIB_ENS_PERSISTENT: lattice and IB phases
- * separated by grid barriers), or by two launches per step (LBIB_ENS_SPLIT:
+ * separated by grid barriers, captured once per step count into a CUDA graph;
+ * the default of one tissue), or by two launches per step (LBIB_ENS_SPLIT:
  * one lattice launch over every node of every tissue, one IB launch over every
- * cell, ordered by programmatic dependent launches; LBIB_ENS_SPLIT_WIDE: the
- * same with more registers and fewer CTAs per SM for the lattice launch),
- * captured once per step count into a CUDA graph.
+ * cell, ordered by programmatic dependent launches; LBIB_ENS_SPLIT_WIDE, the
+ * default of several tissues: the same with more registers and fewer CTAs per
+ * SM for the lattice launch).  A large ensemble runs two groups of tissues
+ * side by side, the second on a stream of the ensemble's own between two
+ * events of the caller's stream.
  * All tissues use LBIB_FP32 storage and share n_species and forcing.  Each
  * tissue is a context: lbib_ensemble_tissue() returns it for
  * lbib_set_cells(), lbib_get_fields(), lbib_get_state() and the like (do not

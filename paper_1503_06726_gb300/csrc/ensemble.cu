@@ -1,4 +1,5 @@
-// ensemble.cu -- a batch of independent tissues advanced together by one
+// ensemble.cu -- a batch of independent tissues advanced together, by two
+// launches per step over all of them (the split schedules) or by one
 // persistent, cooperative kernel launch per lbib_ensemble_step() call.
 //
 // Every tissue is an ordinary context (its own slice of the ensemble's
@@ -6,12 +7,12 @@
 // the per-tissue calls (lbib_set_cells, lbib_get_fields, state) work on it.
 // lbib_ensemble_step(n) runs, for all tissues at once, the same sequence as
 // lbib_step(n): the IB prep, then per step the lattice update of every node
-// of every tissue and the IB move/prep of every cell, separated by grid-wide
-// barriers.  Work is dealt out in items -- lattice items of `nodes_per_item`
+// of every tissue and the IB move/prep of every cell, in the persistent kernel
+// separated by grid-wide barriers.  Work is dealt out in items -- lattice items of `nodes_per_item`
 // nodes (rows padded to 32 so a warp stays in one row) and one item per cell
 // -- strided over the persistent CTAs, which balances tissues of very
-// different sizes.  The launch is captured once per step count into a CUDA
-// graph and replayed.
+// different sizes.  The persistent launch is captured once per step count into
+// a CUDA graph and replayed.
 //
 // The split schedule runs the same items as two kernels per step instead --
 // one lattice launch over every lattice item of every tissue (128-thread
@@ -20,8 +21,8 @@
 // launch over every cell -- ordered by programmatic dependent launches in
 // place of the grid barriers: each kernel issues its loads of what the launch
 // two back wrote before it waits on the launch just before, as the
-// single-tissue steps do.  All 2n + 1 launches of n steps are one graph.
-// The schedule and the two launch parameters (nodes per item, and CTAs per SM
+// single-tissue steps do.  Two groups of tissues run side by side in a large
+// ensemble.  It is the default for two tissues or more.  The schedule and the two launch parameters (nodes per item, and CTAs per SM
 // of the persistent kernel) are chosen by lbib_ensemble_tune(), which times
 // the candidates.
 //
@@ -220,11 +221,11 @@ __global__ void __launch_bounds__(kIBThreads, 3) ensemble_kernel(EnsArgs e) {
 template <int S, int FORCING, bool WIDE>
 __global__ void __launch_bounds__(kLatticeThreads,
                                   LatticeOccupancy<float, S>::kMinBlocks - (WIDE ? 2 : 0))
-    ens_lattice_kernel(EnsArgs e, int step, int out) {
+    ens_lattice_kernel(EnsArgs e, int step, int out, int item0) {
     // the tissue's arguments in shared memory, read from there at each use
     // (held in registers they would spill at the standalone kernel's budget)
     __shared__ TissueDev td;
-    const int item = blockIdx.x;
+    const int item = item0 + blockIdx.x;
     const int t = find_tissue(e.item_pfx, e.n, item);
     {
         const int* src = reinterpret_cast<const int*>(e.tis + t);
@@ -264,13 +265,13 @@ __global__ void __launch_bounds__(kLatticeThreads,
 // tissue (move and/or prep as lbib_step's IB launch, with its programmatic
 // wait on the lattice launch before it).
 template <int NT>
-__global__ void __launch_bounds__(NT) ens_ib_kernel(EnsArgs e, int move, int prep, int vforce) {
+__global__ void __launch_bounds__(NT) ens_ib_kernel(EnsArgs e, int move, int prep, int vforce, int cell0) {
     extern __shared__ __align__(16) unsigned char ens_ib_smem[];
     const IBShared32 view = ib_shared32_view(ens_ib_smem, e.maxv);
     // the tissue's arguments in shared memory (a local copy would live on
     // the stack)
     __shared__ IBArgs ia;
-    const int item = blockIdx.x;
+    const int item = cell0 + blockIdx.x;
     const int t = find_tissue(e.cell_pfx, e.n, item);
     {
         const int* src = reinterpret_cast<const int*>(&e.tis[t].ia);
@@ -311,7 +312,7 @@ static EnsKernel pick_kernel(int S, int forcing) {
     }
 }
 
-typedef void (*EnsLatticeKernel)(EnsArgs, int, int);
+typedef void (*EnsLatticeKernel)(EnsArgs, int, int, int);
 
 template <bool WIDE>
 static EnsLatticeKernel pick_lattice_kernel_w(int S, int forcing) {
@@ -332,6 +333,11 @@ static EnsLatticeKernel pick_lattice_kernel_w(int S, int forcing) {
 static EnsLatticeKernel pick_lattice_kernel(int S, int forcing, bool wide) {
     return wide ? pick_lattice_kernel_w<true>(S, forcing) : pick_lattice_kernel_w<false>(S, forcing);
 }
+
+constexpr int kEnsGroups = 2;  // groups of tissues that run side by side
+// nodes from which two groups are faster than one (us per step with one and
+// two: 0.39 M nodes 20.0 and 20.0, 0.57 M 24.8 and 22.2, 4.4 M 130 and 120)
+constexpr int64_t kEnsGroupNodes = 500000;
 
 static uint64_t up256(uint64_t v) { return (v + 255) / 256 * 256; }
 
@@ -354,6 +360,12 @@ struct lbib_ensemble {
     int n_sms = 0;
     int maxv = 0;           // vertex slots per cell in shared memory (largest cell)
     int schedule = LBIB_ENS_PERSISTENT;
+    // the split schedule's groups of consecutive tissues: where their lattice
+    // items and cells begin (and, last, end)
+    std::vector<int> group_item, group_cell;
+    // the streams and events of the groups after the first
+    cudaStream_t branch[kEnsGroups] = {};
+    cudaEvent_t fork = nullptr, join[kEnsGroups] = {};
     std::map<std::tuple<int, int, int>, cudaGraphExec_t> graphs;
     bool graph_ok = true;
     std::string err;
@@ -439,6 +451,19 @@ static cudaError_t ens_upload(lbib_ensemble* e, int* total_items, int* total_cel
     }
     *total_items = ipfx[e->n];
     *total_cells = cpfx[e->n];
+    // of a large ensemble two groups of about half the nodes each
+    e->group_item.assign(1, 0);
+    e->group_cell.assign(1, 0);
+    const int groups = (int64_t)ipfx[e->n] * e->nodes_per_item >= kEnsGroupNodes ? kEnsGroups : 1;
+    for (int g = 1, t = 0; g < groups; ++g) {
+        while (t < e->n && (int64_t)ipfx[t] * groups < (int64_t)ipfx[e->n] * g) ++t;
+        if (t < e->n && ipfx[t] > e->group_item.back()) {
+            e->group_item.push_back(ipfx[t]);
+            e->group_cell.push_back(cpfx[t]);
+        }
+    }
+    e->group_item.push_back(ipfx[e->n]);
+    e->group_cell.push_back(cpfx[e->n]);
     cudaError_t er = cudaMemcpyAsync(e->ws + e->tab_off, tab.data(), sizeof(TissueDev) * e->n,
                                      cudaMemcpyHostToDevice, e->stream);
     if (er == cudaSuccess)
@@ -492,29 +517,64 @@ static cudaError_t ens_launch(lbib_ensemble* e, const EnsArgs& a, unsigned grid,
     return cudaLaunchKernelEx(&cfg, pick_kernel(e->S, e->forcing), a);
 }
 
-// The split schedule of n steps: the prep, then per step the lattice launch
-// and the IB launch (move, and the prep of the next step but after the last).
-// Every launch after the first is programmatic; without cells the lattice
-// launches follow one another and wait for each other in full.
-static cudaError_t ens_split_enqueue(lbib_ensemble* e, const EnsArgs& a, cudaStream_t st) {
+// The split schedule of n steps for the tissues of group g: the prep, then per
+// step the lattice launch and the IB launch (move, and the prep of the next
+// step but after the last).  Every launch after the first is programmatic;
+// without cells the lattice launches follow one another, each waiting before
+// its first load.
+static cudaError_t ens_split_group(lbib_ensemble* e, const EnsArgs& a, int g, cudaStream_t st) {
+    const int item0 = e->group_item[g], items = e->group_item[g + 1] - item0;
+    const int cell0 = e->group_cell[g], cells = e->group_cell[g + 1] - cell0;
     const size_t smem = ens_cell_smem(a.maxv);
     auto ib = [&](int move, int prep, int vforce, bool pdl) -> cudaError_t {
-        if (a.total_cells == 0) return cudaSuccess;
+        if (cells == 0) return cudaSuccess;
         if (a.cell_threads == 64)
-            return launch_kernel(ens_ib_kernel<64>, dim3(a.total_cells), dim3(64), smem, st, pdl,
-                                 a, move, prep, vforce);
-        return launch_kernel(ens_ib_kernel<128>, dim3(a.total_cells), dim3(128), smem, st, pdl, a,
-                             move, prep, vforce);
+            return launch_kernel(ens_ib_kernel<64>, dim3(cells), dim3(64), smem, st, pdl, a, move,
+                                 prep, vforce, cell0);
+        return launch_kernel(ens_ib_kernel<128>, dim3(cells), dim3(128), smem, st, pdl, a, move,
+                             prep, vforce, cell0);
     };
     const EnsLatticeKernel lk =
         pick_lattice_kernel(e->S, e->forcing, e->schedule == LBIB_ENS_SPLIT_WIDE);
-    const bool pdl = a.total_cells > 0;
     cudaError_t er = ib(0, 1, a.n_steps == 1, false);
     for (int s = 0; s < a.n_steps && er == cudaSuccess; ++s) {
         const bool last = (s == a.n_steps - 1);
-        er = launch_kernel(lk, dim3(a.total_items), dim3(kLatticeThreads), 0, st, pdl, a, s,
-                           last ? 1 : 0);
+        er = launch_kernel(lk, dim3(items), dim3(kLatticeThreads), 0, st, cells > 0 || s > 0, a, s,
+                           last ? 1 : 0, item0);
         if (er == cudaSuccess) er = ib(1, last ? 0 : 1, s == a.n_steps - 2, true);
+    }
+    return er;
+}
+
+// The split schedule.  The tissues are independent, so while one group's IB
+// launch, which waits on memory latency, leaves the DRAM idle, another
+// group's lattice launch uses it: the groups run on streams of their own
+// between two events of the ensemble's stream (30 tissues of 128^2 .. 1024^2:
+// 217 -> 202 us per step).  Launched one by one (3 us of host time per step):
+// replayed from a graph the same launches took 15.2 us per step for two small
+// tissues against 13.1.
+static cudaError_t ens_split_enqueue(lbib_ensemble* e, const EnsArgs& a, cudaStream_t st) {
+    const int groups = (int)e->group_item.size() - 1;
+    cudaError_t er = cudaSuccess;
+    if (groups > 1) {
+        if (!e->fork) er = cudaEventCreateWithFlags(&e->fork, cudaEventDisableTiming);
+        if (er == cudaSuccess) er = cudaEventRecord(e->fork, st);
+    }
+    for (int g = 1; g < groups && er == cudaSuccess; ++g) {
+        if (!e->branch[g]) er = cudaStreamCreateWithFlags(&e->branch[g], cudaStreamNonBlocking);
+        if (er == cudaSuccess && !e->join[g])
+            er = cudaEventCreateWithFlags(&e->join[g], cudaEventDisableTiming);
+        if (er == cudaSuccess) er = cudaStreamWaitEvent(e->branch[g], e->fork, 0);
+    }
+    // (both groups' launches in turn would keep the host nearer to both
+    // streams; a group's launches are a few microseconds each, its steps tens)
+    for (int g = 0; g < groups && er == cudaSuccess; ++g)
+        er = ens_split_group(e, a, g, g ? e->branch[g] : st);
+    // whatever was enqueued on the branches ends before the stream goes on
+    for (int g = 1; g < groups && e->join[g]; ++g) {
+        const cudaError_t e1 = cudaEventRecord(e->join[g], e->branch[g]);
+        const cudaError_t e2 = cudaStreamWaitEvent(st, e->join[g], 0);
+        if (er == cudaSuccess) er = e1 != cudaSuccess ? e1 : e2;
     }
     return er;
 }
@@ -608,6 +668,17 @@ int lbib_ensemble_create(int32_t n, const lbib_params* params, const int32_t* ma
         return ens_fail(nullptr, LBIB_E_CUDA,
                         std::string("lbib_ensemble_create: ") + cudaGetErrorString(er));
     }
+    // several tissues: the split schedule with the lattice kernel that does not
+    // spill was the fastest at every size measured (us per step against the
+    // persistent kernel's: 2 tissues of 64^2 .. 220^2 13.1 against 23.6, 30 of
+    // 100^2 .. 300^2 34 against 57, 30 of 128^2 .. 1024^2 202 against 268, 64 of
+    // them 423 against 540), with 256 nodes per CTA below 0.8 M nodes (16
+    // tissues, 0.57 M: 22.2 us against 26.7) and 512 above (30 tissues, 1.1 M:
+    // 33.9 against 36.6).  One tissue starts with the persistent kernel.
+    int64_t nodes = 0;
+    for (int t = 0; t < n; ++t) nodes += (int64_t)params[t].nx * params[t].ny;
+    if (n > 1) e->schedule = LBIB_ENS_SPLIT_WIDE;
+    if (nodes >= 800000) e->nodes_per_item = 512;
     *out = e;
     return LBIB_OK;
 }
@@ -631,12 +702,13 @@ int lbib_ensemble_step(lbib_ensemble* e, int32_t n_steps) {
         return ens_fail(e, LBIB_E_CUDA, std::string("lbib_ensemble_step: ") + cudaGetErrorString(er));
     const unsigned grid = ens_grid(e);
     const EnsArgs a = ens_args(e, n_steps, items, cells, grid);
-    // the kernel reads the table at run time; the graph depends only on the
-    // step count, the launch shape and the work totals
+    // the persistent kernel reads the table at run time; its graph depends only
+    // on the step count, the launch shape and the work totals
     const auto key = std::make_tuple((int)n_steps, items, cells);
+    const bool persistent = e->schedule == LBIB_ENS_PERSISTENT;
     auto it = e->graphs.find(key);
     bool launched = false;
-    if (e->graph_ok && it == e->graphs.end()) {
+    if (persistent && e->graph_ok && it == e->graphs.end()) {
         cudaStream_t cap;
         er = cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking);
         cudaGraph_t g = nullptr;
@@ -657,7 +729,7 @@ int lbib_ensemble_step(lbib_ensemble* e, int32_t n_steps) {
             e->graph_ok = false;  // fall back to direct launches
         }
     }
-    if (e->graph_ok && it != e->graphs.end()) {
+    if (persistent && e->graph_ok && it != e->graphs.end()) {
         er = cudaGraphLaunch(it->second, e->stream);
         launched = true;
     }
@@ -820,6 +892,11 @@ int lbib_ensemble_selftest_timeout(lbib_ensemble* e, double* seconds_out) {
 void lbib_ensemble_destroy(lbib_ensemble* e) {
     if (!e) return;
     ens_drop_graphs(e);
+    for (int g = 0; g < kEnsGroups; ++g) {
+        if (e->branch[g]) cudaStreamDestroy(e->branch[g]);
+        if (e->join[g]) cudaEventDestroy(e->join[g]);
+    }
+    if (e->fork) cudaEventDestroy(e->fork);
     for (auto* c : e->ctx) lbib_destroy(c);
     delete e;
 }
