@@ -752,4 +752,46 @@ cudaError_t launch_set_species(int precision, int n_species, int s_idx, int nx, 
     return cudaGetLastError();
 }
 
+// ---------------------------------------------------------------------------
+// An output field for the host: rows [y0, y1) of a plane, packed, as doubles
+// (labels: the packed word as 0 outside, cell + 1 inside).  A plane of pairs
+// (velocity, force) gives one component with step 2, both with step 1 and
+// twice the columns.
+template <typename C>
+__global__ void unpack_kernel(const C* plane, int64_t pitch, int nx, int step, int first,
+                              double* out) {
+    const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t y = blockIdx.y;
+    if (x < nx) out[y * nx + x] = (double)plane[(y * pitch + x) * step + first];
+}
+__global__ void unpack_ids_kernel(const uint32_t* plane, int64_t pitch, int nx, int32_t* out) {
+    const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t y = blockIdx.y;
+    if (x >= nx) return;
+    const uint32_t v = plane[y * pitch + x];
+    out[y * nx + x] = v == kOutside ? 0 : (int32_t)(v >> 4) + 1;
+}
+
+cudaError_t launch_unpack(int cs, const void* plane, int64_t pitch, int nx, int y0, int y1,
+                          int step, int first, void* out, cudaStream_t s) {
+    for (int y = y0; y < y1;) {  // (a grid has at most 65,535 rows)
+        const int n = y1 - y < 65535 ? y1 - y : 65535;
+        const dim3 grid((nx + 255) / 256, n), block(256);
+        const int64_t o = (int64_t)(y - y0) * nx, at = y * pitch * step;
+        if (cs == 8)
+            unpack_kernel<<<grid, block, 0, s>>>(static_cast<const double*>(plane) + at, pitch, nx,
+                                                 step, first, static_cast<double*>(out) + o);
+        else if (cs == 4)
+            unpack_kernel<<<grid, block, 0, s>>>(static_cast<const float*>(plane) + at, pitch, nx,
+                                                 step, first, static_cast<double*>(out) + o);
+        else
+            unpack_ids_kernel<<<grid, block, 0, s>>>(static_cast<const uint32_t*>(plane) + at,
+                                                     pitch, nx, static_cast<int32_t*>(out) + o);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+        y += n;
+    }
+    return cudaSuccess;
+}
+
 }  // namespace lbib

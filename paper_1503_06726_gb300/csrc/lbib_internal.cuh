@@ -156,6 +156,10 @@ struct Layout {
     int jnbx = 0, jnby = 0;
     // FP64 conservation sums (lbib_get_sums): global, per cell, non-finite count
     uint64_t sums = 0, sums_bytes = 0;
+    // FP64 staging of rows of a lattice field on their way to the host (large
+    // lattices; 0 bytes for small ones)
+    uint64_t stage = 0;
+    uint64_t stage_bytes = 0;
     uint64_t diag = 0;
     uint64_t total = 0;
 };
@@ -526,6 +530,11 @@ cudaError_t launch_make_ncode(const int32_t* dom, uint16_t* ncode, int nx, int n
                               int64_t pitch, cudaStream_t s);
 // the species moments (phi, jx, jy per species; compute type) of the stored
 // populations g at every node (the moments a run starts from)
+// rows [y0, y1) of an output plane of the compute type (cs bytes) as
+// packed doubles, or of the labels (cs 0) as packed int32: element `first` of
+// every `step` (the planes of pairs), see unpack_kernel
+cudaError_t launch_unpack(int cs, const void* plane, int64_t pitch, int nx, int y0, int y1,
+                          int step, int first, void* out, cudaStream_t s);
 cudaError_t launch_species_moments(int precision, int n_species, int nx, int ny, int64_t pitch,
                                    int64_t plane, const void* g, void* mom, const void* coefs,
                                    cudaStream_t s);
