@@ -79,6 +79,21 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
     return (uint32_t)__cvta_generic_to_shared(p);
 }
 
+// One lane of a converged warp, the same one every time.  The tensor core
+// instructions are issued under it rather than under a test of the thread
+// index: their operands live in uniform registers, and only where the compiler
+// knows that one lane runs does it keep them there.  256^2, 16 images, 32 -> 32
+// channels: weight gradient 116 us (descriptors built anew for each multiply)
+// -> 101 (by increments) -> 75 (elected lane), forward 62 -> 60 -> 50; the
+// decoder's 80 -> 32 channels 379 -> 333 -> 251 and 222 -> 187 -> 141.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile(
+        "{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(p));
+    return p != 0;
+}
+
 // ---- mbarriers
 __device__ __forceinline__ void mbar_init(uint32_t a, uint32_t count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(a), "r"(count) : "memory");
@@ -177,15 +192,20 @@ __host__ __device__ __forceinline__ uint32_t swizzle_off(uint32_t off, int swb) 
 __device__ __forceinline__ void expand_upsampled(unsigned char* dst, const unsigned char* stg,
                                                  int halo_rows, int rs, int swb, int x0, int y0,
                                                  int up_cols, int tid, int nthreads) {
-    const int ppp = swb / 16;
+    const int sh = swb == 64 ? 2 : (swb == 32 ? 1 : 3);  // 16-byte pieces of a pixel: 1 << sh
     const int by = (y0 - 1) >> 1, bx = (x0 - 1) >> 1;
-    for (int i = tid; i < halo_rows * rs * ppp; i += nthreads) {
-        const int hp = i / ppp, q = i % ppp;
-        const int gy = y0 - 1 + hp / rs, gx = x0 - 1 + hp % rs;
-        const int srow = ((gy >> 1) - by) * up_cols + ((gx >> 1) - bx);
+    const int width = rs << sh;  // pieces of a halo row
+    int r = 0, j = tid;
+    while (j >= width) j -= width, ++r;
+    for (; r < halo_rows;) {
+        const int c = j >> sh, q = j & ((1 << sh) - 1);
+        const int srow = (((y0 - 1 + r) >> 1) - by) * up_cols + (((x0 - 1 + c) >> 1) - bx);
         const uint4 v = *reinterpret_cast<const uint4*>(
             stg + swizzle_off((uint32_t)(srow * swb + q * 16), swb));
-        *reinterpret_cast<uint4*>(dst + swizzle_off((uint32_t)(hp * swb + q * 16), swb)) = v;
+        *reinterpret_cast<uint4*>(
+            dst + swizzle_off((uint32_t)((r * rs + c) * swb + q * 16), swb)) = v;
+        j += nthreads;
+        while (j >= width) j -= width, ++r;
     }
 }
 // Instruction descriptor of kind::f16: FP32 accumulator (bits 4-5 = 1), BF16
@@ -203,10 +223,30 @@ __device__ __forceinline__ void tc_mma(uint32_t d_tmem, uint64_t adesc, uint64_t
         "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
         : "memory");
 }
+// the same, always adding
+__device__ __forceinline__ void tc_mma_add(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc,
+                                           uint32_t idesc) {
+    asm volatile(
+        "{\n .reg .pred p;\n setp.eq.b32 p, 0, 0;\n"
+        " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
+        "l"(adesc), "l"(bdesc), "r"(idesc)
+        : "memory");
+}
 __device__ __forceinline__ void tc_commit(uint32_t mbar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::
                      "r"(mbar)
                  : "memory");
+}
+// 16 accumulator columns of the warp's lanes; the loads of several calls run
+// together until tmem_wait
+__device__ __forceinline__ void tmem_ld16_start(uint32_t taddr, uint32_t* r) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,"
+        "%14,%15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+          "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]),
+          "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr));
 }
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float v[16]) {
     uint32_t r[16];
@@ -223,6 +263,44 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float v[16]) {
 }
 
 
+// The multiplies of one chunk: nine taps, KK steps of 16 channels, M
+// accumulators, unrolled (a multiply of 128 x 32 x 16 takes the tensor core
+// little longer than its issue).
+template <int KK, int M>
+__device__ __forceinline__ void issue_taps(uint64_t a0, uint64_t b0, uint32_t tmem, uint32_t idesc,
+                                           const ConvTcArgs& a, bool more) {
+    constexpr uint32_t pixel = 2u * KK;  // 16-byte units of a pixel
+    const uint32_t jstep = (uint32_t)(a.wide ? a.rs : kTcM) * pixel;
+    const uint32_t bstep = (uint32_t)a.Np * pixel, Np = (uint32_t)a.Np;
+#pragma unroll
+    for (int t = 0; t < 9; ++t) {
+        const uint32_t at = ((uint32_t)(t / 3 * a.rs) + t % 3) * pixel;
+#pragma unroll
+        for (int kk = 0; kk < KK; ++kk) {
+            const uint64_t ad = a0 + at + 2 * kk, bd = b0 + t * bstep + 2 * kk;
+#pragma unroll
+            for (int j = 0; j < M; ++j) {
+                if (t == 0 && kk == 0)
+                    tc_mma(tmem + j * Np, ad + j * jstep, bd, idesc, more ? 1u : 0u);
+                else
+                    tc_mma_add(tmem + j * Np, ad + j * jstep, bd, idesc);
+            }
+        }
+    }
+}
+template <int KK>
+__device__ __forceinline__ void issue_chunk(uint64_t a0, uint64_t b0, uint32_t tmem, uint32_t idesc,
+                                            const ConvTcArgs& a, bool more) {
+    if (a.m == 4)
+        issue_taps<KK, 4>(a0, b0, tmem, idesc, a, more);
+    else if (a.m == 3)
+        issue_taps<KK, 3>(a0, b0, tmem, idesc, a, more);
+    else if (a.m == 2)
+        issue_taps<KK, 2>(a0, b0, tmem, idesc, a, more);
+    else
+        issue_taps<KK, 1>(a0, b0, tmem, idesc, a, more);
+}
+
 // UP: the layer has upsampled channels (the expansion is compiled only then)
 template <bool UP>
 __global__ void __launch_bounds__(kTcThreads)
@@ -232,6 +310,7 @@ __global__ void __launch_bounds__(kTcThreads)
     __shared__ __align__(8) uint64_t bar_full[kTcMaxStages], bar_done[kTcMaxStages];
     __shared__ uint32_t tmem_slot;
     __shared__ int s_bad, s_committed, s_up_ok;
+    __shared__ float s_bias[192];
     // stages at 1024-byte boundaries: the swizzle follows the address bits
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -244,6 +323,8 @@ __global__ void __launch_bounds__(kTcThreads)
     const int co0 = blockIdx.y * a.Np;  // this CTA's output channels
     const __nv_bfloat16* wt = a.wt + (int64_t)blockIdx.y * a.nk * 9 * a.Np * a.Kc;
 
+    for (int c = tid; c < a.Np; c += kTcThreads)
+        s_bias[c] = a.bias && co0 + c < a.Co ? a.bias[co0 + c] : 0.f;
     if (tid == 0) {
         for (int s = 0; s < NS; ++s) {
             mbar_init(smem_u32(&bar_full[s]), 1);
@@ -263,13 +344,12 @@ __global__ void __launch_bounds__(kTcThreads)
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = tmem_slot;
+    const uint32_t tmem = __shfl_sync(0xffffffffu, tmem_slot, 0);
     const uint32_t idesc = mma_idesc(kTcM, a.Np);
     const uint32_t b_bytes = 9u * (uint32_t)a.Np * (uint32_t)a.swb;
     const uint32_t sbo = 8u * (uint32_t)a.swb;
-    // thread 0: per stage, the chunk whose copies were issued and not yet
-    // waited for (-1 = none)
-    int loading[kTcMaxStages] = {-1, -1, -1};
+    // the issuing thread: chunks whose copies were issued, and waited for
+    int issued = 0, landed = 0;
 
     auto issue = [&](int k) {
         const int s = k % NS;
@@ -284,7 +364,7 @@ __global__ void __launch_bounds__(kTcThreads)
                         (y0 - 1) >> 1, n, fb);
         }
         bulk_load(st + (uint32_t)a.a_bytes, wt + (int64_t)k * 9 * a.Np * a.Kc, b_bytes, fb);
-        loading[s] = k;
+        issued = k + 1;
     };
 
     // an upsampled chunk: once its half-resolution box has landed the threads
@@ -308,7 +388,7 @@ __global__ void __launch_bounds__(kTcThreads)
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     };
 
-    if (tid == 0)
+    if (warp == 0 && elect_one())
         for (int k = 0; k < NS && k < a.nk; ++k) issue(k);
     if (UP && a.nk1 == 0) {
         expand_chunk(0);
@@ -317,27 +397,22 @@ __global__ void __launch_bounds__(kTcThreads)
     for (int k = 0; k < a.nk; ++k) {
         const int s = k % NS;
         const uint32_t st = base + (uint32_t)s * (uint32_t)a.stage_bytes;
-        if (tid == 0) {
+        if (warp == 0 && elect_one()) {
             if (!mbar_wait(smem_u32(&bar_full[s]), (k / NS) & 1)) {
                 s_bad = 1;
             } else {
-                loading[s] = -1;
+                landed = k + 1;
                 tc_fence_after();
-                const uint32_t bst = st + (uint32_t)a.a_bytes;
-                for (int t = 0; t < 9; ++t) {
-                    const int ky = t / 3, kx = t % 3;
-                    for (int kk = 0; kk < a.Kc / 16; ++kk) {
-                        const uint64_t bdesc = smem_desc_sw(
-                            bst + (uint32_t)(t * a.Np * a.swb + kk * 32), sbo, (uint32_t)a.swcode);
-                        for (int j = 0; j < a.m; ++j) {
-                            const int row = (a.wide ? j * a.rs : j * kTcM) + ky * a.rs + kx;
-                            const uint64_t adesc = smem_desc_sw(
-                                st + (uint32_t)(row * a.swb + kk * 32), sbo, (uint32_t)a.swcode);
-                            tc_mma(tmem + (uint32_t)(j * a.Np), adesc, bdesc, idesc,
-                                   (k > 0 || t > 0 || kk > 0) ? 1u : 0u);
-                        }
-                    }
-                }
+                // the descriptors of later rows, taps and chunks are the first
+                // ones' plus their distance in 16-byte units (the address is
+                // the low field, and shared memory ends below its range)
+                const uint64_t a0 = smem_desc_sw(st, sbo, (uint32_t)a.swcode);
+                const uint64_t b0 =
+                    smem_desc_sw(st + (uint32_t)a.a_bytes, sbo, (uint32_t)a.swcode);
+                if (a.Kc == 32)
+                    issue_chunk<2>(a0, b0, tmem, idesc, a, k > 0);
+                else
+                    issue_chunk<1>(a0, b0, tmem, idesc, a, k > 0);
                 tc_commit(smem_u32(&bar_done[s]));
                 s_committed = k;
                 // refill the stage of chunk k - 1, whose multiplies ran ahead
@@ -355,9 +430,9 @@ __global__ void __launch_bounds__(kTcThreads)
         if (s_bad) break;
     }
     // after an error: the copies still in flight land before the CTA leaves
-    if (tid == 0)
-        for (int s = 0; s < NS; ++s)
-            if (loading[s] >= 0) mbar_wait(smem_u32(&bar_full[s]), (loading[s] / NS) & 1);
+    if (warp == 0 && elect_one())
+        for (int k = landed; k < issued; ++k)
+            mbar_wait(smem_u32(&bar_full[k % NS]), (k / NS) & 1);
     __syncthreads();
     // the last commit covers every multiply issued before it
     const int committed = s_committed;
@@ -370,65 +445,84 @@ __global__ void __launch_bounds__(kTcThreads)
         // epilogue: warp w owns lanes 32w .. 32w + 31 of every accumulator
         const int i = warp * 32 + lane;
         const uint32_t trow = tmem + ((uint32_t)(warp * 32) << 16);
+        // groups of 16 channels move as 16-byte words where the channel count
+        // allows (out and gate are 16-byte aligned)
+        const bool words = a.Co % 8 == 0;
         for (int j = 0; j < a.m; ++j) {
             const int lin = j * kTcM + i;
             const int r = a.wide ? j : lin / a.rs, c = a.wide ? i : lin % a.rs;
             const bool valid = c < a.Wt && r < a.TR && y0 + r < a.H;
             const int64_t pix = ((int64_t)n * a.H + y0 + r) * a.W + x0 + c;
-            for (int cl = 0; cl < a.Np; cl += 16) {
-                float v[16];
-                tmem_ld16(trow + (uint32_t)(j * a.Np + cl), v);
-                if (!valid) continue;
-                const int c0 = co0 + cl;
-#pragma unroll
-                for (int q = 0; q < 16; ++q) {
-                    const int co = c0 + q;
-                    if (co < a.Co) {
-                        if (a.bias) v[q] += a.bias[co];
-                        if (a.relu) v[q] = fmaxf(v[q], 0.f);
-                    }
+            for (int cl = 0; cl < a.Np; cl += 32) {
+                // up to 32 columns and their gates in flight at once
+                const bool two = cl + 16 < a.Np;
+                uint32_t r32[32];
+                __syncwarp();
+                tmem_ld16_start(trow + (uint32_t)(j * a.Np + cl), r32);
+                if (two) tmem_ld16_start(trow + (uint32_t)(j * a.Np + cl + 16), r32 + 16);
+                uint4 gt4[4];
+                if (a.gate && words && valid) {
+                    const uint4* gt =
+                        reinterpret_cast<const uint4*>(a.gate + pix * a.Co + co0 + cl);
+                    if (co0 + cl + 16 <= a.Co) gt4[0] = __ldg(gt), gt4[1] = __ldg(gt + 1);
+                    if (two && co0 + cl + 32 <= a.Co)
+                        gt4[2] = __ldg(gt + 2), gt4[3] = __ldg(gt + 3);
                 }
-                if (a.gate) {
-                    const __nv_bfloat16* gt = a.gate + pix * a.Co + c0;
-                    if (c0 + 16 <= a.Co && (a.Co % 8) == 0) {
-                        __nv_bfloat162 h[8];
-                        const uint4 g0 = __ldg(reinterpret_cast<const uint4*>(gt));
-                        const uint4 g1 = __ldg(reinterpret_cast<const uint4*>(gt) + 1);
-                        std::memcpy(&h[0], &g0, 16);
-                        std::memcpy(&h[4], &g1, 16);
+                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                if (!valid) continue;
 #pragma unroll
-                        for (int q = 0; q < 8; ++q) {
-                            const float2 f = __bfloat1622float2(h[q]);
-                            if (!(f.x > 0.f)) v[2 * q] = 0.f;
-                            if (!(f.y > 0.f)) v[2 * q + 1] = 0.f;
+                for (int h = 0; h < 2; ++h) {
+                    const int c0 = co0 + cl + 16 * h;
+                    if ((h && !two) || c0 >= a.Co) break;
+                    float v[16];
+#pragma unroll
+                    for (int q = 0; q < 16; ++q)
+                        v[q] = __uint_as_float(r32[16 * h + q]) + s_bias[cl + 16 * h + q];
+                    if (a.relu) {
+#pragma unroll
+                        for (int q = 0; q < 16; ++q) v[q] = fmaxf(v[q], 0.f);
+                    }
+                    if (words && c0 + 16 <= a.Co) {
+                        if (a.gate) {
+                            __nv_bfloat162 g[8];
+                            std::memcpy(&g[0], &gt4[2 * h], 32);
+#pragma unroll
+                            for (int q = 0; q < 8; ++q) {
+                                const float2 f = __bfloat1622float2(g[q]);
+                                if (!(f.x > 0.f)) v[2 * q] = 0.f;
+                                if (!(f.y > 0.f)) v[2 * q + 1] = 0.f;
+                            }
+                        }
+                        if (a.out_f32) {
+                            float4* o = reinterpret_cast<float4*>(static_cast<float*>(a.out) +
+                                                                  pix * a.Co + c0);
+#pragma unroll
+                            for (int q = 0; q < 4; ++q)
+                                o[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2],
+                                                   v[4 * q + 3]);
+                        } else {
+                            __nv_bfloat162 b[8];
+                            uint4 w[2];
+#pragma unroll
+                            for (int q = 0; q < 8; ++q)
+                                b[q] = __floats2bfloat162_rn(v[2 * q], v[2 * q + 1]);
+                            std::memcpy(&w[0], &b[0], 32);
+                            uint4* o = reinterpret_cast<uint4*>(
+                                static_cast<__nv_bfloat16*>(a.out) + pix * a.Co + c0);
+                            o[0] = w[0];
+                            o[1] = w[1];
                         }
                     } else {
 #pragma unroll
-                        for (int q = 0; q < 16; ++q)
-                            if (c0 + q < a.Co && !(__bfloat162float(gt[q]) > 0.f)) v[q] = 0.f;
-                    }
-                }
-                if (a.out_f32) {
-                    float* o = static_cast<float*>(a.out) + pix * a.Co;
-#pragma unroll
-                    for (int q = 0; q < 16; ++q)
-                        if (c0 + q < a.Co) o[c0 + q] = v[q];
-                } else {
-                    __nv_bfloat16* o = static_cast<__nv_bfloat16*>(a.out) + pix * a.Co + c0;
-                    if (c0 + 16 <= a.Co && (a.Co % 8) == 0) {
-                        uint4 w0, w1;
-                        __nv_bfloat162 h[8];
-#pragma unroll
-                        for (int q = 0; q < 8; ++q)
-                            h[q] = __floats2bfloat162_rn(v[2 * q], v[2 * q + 1]);
-                        std::memcpy(&w0, &h[0], 16);
-                        std::memcpy(&w1, &h[4], 16);
-                        reinterpret_cast<uint4*>(o)[0] = w0;
-                        reinterpret_cast<uint4*>(o)[1] = w1;
-                    } else {
-#pragma unroll
-                        for (int q = 0; q < 16; ++q)
-                            if (c0 + q < a.Co) o[q] = __float2bfloat16_rn(v[q]);
+                        for (int q = 0; q < 16; ++q) {
+                            if (c0 + q >= a.Co) break;
+                            const int64_t at = pix * a.Co + c0 + q;
+                            if (a.gate && !(__bfloat162float(a.gate[at]) > 0.f)) v[q] = 0.f;
+                            if (a.out_f32)
+                                static_cast<float*>(a.out)[at] = v[q];
+                            else
+                                static_cast<__nv_bfloat16*>(a.out)[at] = __float2bfloat16_rn(v[q]);
+                        }
                     }
                 }
             }
@@ -475,18 +569,24 @@ __global__ void tile_weights_tc_kernel(const __nv_bfloat16* w, int Co, int Ci, i
 // pixels p of X[p + (ky - 1, kx - 1)][ci] G[p][co], a GEMM with the pixels as
 // K.  Both operands are staged as pixel rows (channels contiguous), so they
 // enter the MMA MN-major: A rows (M) are input channels, B rows (N) output
-// channels, K runs down the pixel rows.  The X halo of a tile (TR + 2 rows of
-// rs = Wt + 2 pixels, one Kc-channel chunk, swizzled as in the forward
-// kernel) makes every tap a row-shifted window, and the MN-major A operand
-// puts four such windows side by side: its M atoms (Kc channels each) sit one
-// pixel row apart (LBO = one row), so M = 128 covers the taps kx = 0, 1, 2
-// (and a fourth, unused shift) of one ky for 32 channels -- with 16-channel
-// chunks eight shifts, three of them used.  The K steps walk the tile's image
-// rows 16 pixels at a time (Wt a multiple of 16), so the halo columns never
-// enter: G is staged without halo, 16 output channels per TMA box (32-byte
-// swizzle), its N atoms a region apart.  One accumulator per ky and per
-// "set" of image rows (rows r % sets; more independent accumulation chains
-// in flight), summed at the end and added to dW with FP32 reductions.  A CTA
+// channels, K runs down the pixel rows.  The X tile (TR rows of rs = Wt + 2
+// pixels, one Kc-channel chunk, swizzled as in the forward kernel) makes every
+// kx a row-shifted window, and the MN-major A operand puts four such windows
+// side by side: its M atoms (Kc channels each) sit one pixel row apart (LBO =
+// one row), so M = 128 covers the taps kx = 0, 1, 2 (and a fourth, unused
+// shift) for 32 channels -- with 16-channel chunks eight shifts, three of them
+// used.  G is staged with a halo of one image row on either side, each row as
+// 16-channel atoms of Wt pixels (32-byte swizzle, one TMA box each), so that
+// the rows y - 1, y, y + 1 that pair with X row y (ky = 2, 1, 0) follow each
+// other and are one operand of N = 3 Np: a multiply costs about 53 + 1.7 N
+// cycles here, most of it the A operand at small N, and one takes the place of
+// three (256^2, 16 images: 32 -> 32 channels 75 us with one row at a time, 61
+// with three; 80 -> 32 251 and 189).  Where 3 Np exceeds the largest N of 256,
+// the first two or one, then the others (the network's levels of 32^2 and 16^2:
+// 19 us, and 18 with one row at a time and no halo of G).  The K steps walk the tile's image rows 16 pixels at a time (Wt a
+// multiple of 16), so the halo columns never enter.  One accumulator per
+// "set" of image rows (rows r % sets; more independent accumulation chains in
+// flight), summed at the end and added to dW with FP32 reductions.  A CTA
 // takes one input-channel chunk, one N tile and a range of pixel tiles
 // (split K over CTAs).  Pipeline and bounded waits as the forward kernel.
 constexpr int kTcMaxChunks = 24;  // input-channel chunks of a weight gradient (up to 384 channels)
@@ -508,11 +608,26 @@ struct WgTcArgs {
     int Wt, rs, TR, tiles_x, tiles_y, total_tiles;
     int sk;                    // CTAs sharing one (chunk, N tile): split K
     int sets;                  // accumulator sets
-    int x_bytes, x_box_bytes;  // the X halo region of a stage, one TMA box
-    int g_atom_bytes;          // one G atom region (TR Wt 32 bytes)
+    int x_bytes;               // the X region of a stage
+    int g_atom_bytes;          // one G atom: 16 channels of an image row (Wt 32 bytes)
     int stage_bytes, stages, tmem_cols;
     int up_rows, up_cols, up_off, up_box_bytes;  // the half-resolution box, as in ConvTcArgs
 };
+
+// the steps of an X row where its three G rows are no single operand: `lead`
+// (1 or 2) of them, then the others
+__device__ __forceinline__ void issue_row(uint32_t d, uint32_t Np, uint64_t xd, uint32_t xstep,
+                                          uint64_t gd, uint32_t grow, uint32_t idesc,
+                                          uint32_t idesc1, int lead, uint32_t acc, int steps) {
+    for (int i = 0; i < steps; ++i) {
+        tc_mma(d, xd, gd, idesc, acc);
+        if (lead == 1) tc_mma(d + Np, xd, gd + grow, idesc1, acc);
+        tc_mma(d + 2 * Np, xd, gd + 2 * grow, idesc1, acc);
+        xd += xstep;
+        gd += 32;
+        acc = 1u;
+    }
+}
 
 template <bool UP>
 __global__ void __launch_bounds__(kTcThreads, 1)
@@ -525,6 +640,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     __shared__ __align__(8) uint64_t bar_full[kTcMaxStages], bar_done[kTcMaxStages];
     __shared__ uint32_t tmem_slot;
     __shared__ int s_bad, s_committed, s_up_ok;
+    __shared__ float s_db[160];
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int NS = a.stages;
@@ -537,7 +653,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     const bool up = UP && a.ck_up[chunk] != 0;  // the chunk comes from the upsampled input
     const CUtensorMap* mapx = Kc == 32 ? &mapx32 : &mapx16;
     const CUtensorMap* mapu = Kc == 32 ? &mapu32 : &mapu16;
-    const uint32_t x_box_bytes = (uint32_t)((a.TR + 2) * a.rs * swx);
+    const uint32_t x_box_bytes = (uint32_t)(a.TR * a.rs * swx);
     const uint32_t up_box_bytes = (uint32_t)(a.up_rows * a.up_cols * swx);
     // this CTA's pixel tiles
     const int t_begin = (int)((int64_t)a.total_tiles * blockIdx.x / a.sk);
@@ -564,16 +680,27 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = tmem_slot;
-    // M = 128 (the Kc-channel atoms of natoms shifts), N = Np, both MN-major
-    const uint32_t idesc = mma_idesc(kTcM, a.Np) | (1u << 15) | (1u << 16);
-    const uint32_t g_bytes = (uint32_t)a.ng * (uint32_t)a.g_atom_bytes;
-    int loading[kTcMaxStages] = {-1, -1, -1};
-    uint32_t started = 0u;  // accumulators that hold a first product
+    const uint32_t tmem = __shfl_sync(0xffffffffu, tmem_slot, 0);
+    // M = 128 (the Kc-channel atoms of the shifts), N = Np for each of the
+    // `lead` rows of the first multiply of a step, both MN-major
+    const int lead = 3 * a.Np <= 256 ? 3 : (2 * a.Np <= 256 ? 2 : 1);
+    const uint32_t idesc = mma_idesc(kTcM, lead * a.Np) | (1u << 15) | (1u << 16);
+    const uint32_t idesc1 = mma_idesc(kTcM, a.Np) | (1u << 15) | (1u << 16);
+    const uint32_t g_row = (uint32_t)a.ng * (uint32_t)a.g_atom_bytes;  // an image row of G
+    const uint32_t g_bytes = (uint32_t)(a.TR + 2) * g_row;
+    int issued = 0, landed = 0;  // the issuing thread: tiles whose copies were issued, waited for
     // the CTAs of the first chunk also sum the bias gradient, in warps 1 - 3
-    // (warp 0 issues the multiplies): channels tid - 32 and tid + 64 of the N tile
-    const bool dbsum = a.db != nullptr && chunk == 0 && tid >= 32 && tid - 32 < a.Np;
-    float db_acc[2] = {0.f, 0.f};
+    // (warp 0 issues the multiplies): 48 / ng pairs of threads per G atom, each
+    // thread 8 channels (one 16-byte piece) of every (48 / ng)-th pixel.  (With
+    // one thread per channel over all pixels this takes longer than the
+    // multiplies: 256^2, 16 images, 32 -> 32 channels 81 us against 75.)
+    const int db_phases = 48 / a.ng;
+    const int db_atom = ((tid - 32) >> 1) / db_phases;
+    const int db_phase = ((tid - 32) >> 1) % db_phases;
+    const int db_half = tid & 1;
+    const bool dbsum = a.db != nullptr && chunk == 0 && tid >= 32 && db_atom < a.ng;
+    float db_acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    for (int c = tid; c < a.Np; c += kTcThreads) s_db[c] = 0.f;
 
     auto tile_xy = [&](int T, int& n, int& y0, int& x0) {
         n = T / per_img;
@@ -589,15 +716,17 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         tile_xy(t_begin + k, n, y0, x0);
         if (!up) {
             mbar_expect_tx(fb, g_bytes + x_box_bytes);
-            tma_load_4d(st, mapx, c0, x0 - 1, y0 - 1, n, fb);
+            tma_load_4d(st, mapx, c0, x0 - 1, y0, n, fb);
         } else {
             mbar_expect_tx(fb, g_bytes + up_box_bytes);
-            tma_load_4d(st + (uint32_t)a.up_off, mapu, c0, (x0 - 1) >> 1, (y0 - 1) >> 1, n, fb);
+            tma_load_4d(st + (uint32_t)a.up_off, mapu, c0, (x0 - 1) >> 1, y0 >> 1, n, fb);
         }
-        for (int at = 0; at < a.ng; ++at)
-            tma_load_4d(st + (uint32_t)a.x_bytes + (uint32_t)(at * a.g_atom_bytes), &mapg,
-                        co0 + 16 * at, x0, y0, n, fb);
-        loading[s] = k;
+        for (int r = 0; r < a.TR + 2; ++r)  // (rows outside the image: zeros)
+            for (int at = 0; at < a.ng; ++at)
+                tma_load_4d(st + (uint32_t)a.x_bytes + (uint32_t)r * g_row +
+                                (uint32_t)(at * a.g_atom_bytes),
+                            &mapg, co0 + 16 * at, x0, y0 - 1 + r, n, fb);
+        issued = k + 1;
     };
 
     // an upsampled chunk: each tile's half-resolution box expanded into the
@@ -614,13 +743,13 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         __syncthreads();
         if (s_up_ok && mbar_wait(smem_u32(&bar_full[s]), (k / NS) & 1)) {
             unsigned char* gst = smem_raw + (st - smem_u32(smem_raw));
-            expand_upsampled(gst, gst + a.up_off, a.TR + 2, a.rs, swx, x0, y0, a.up_cols, tid,
+            expand_upsampled(gst, gst + a.up_off, a.TR, a.rs, swx, x0, y0 + 1, a.up_cols, tid,
                              kTcThreads);
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     };
 
-    if (tid == 0)
+    if (warp == 0 && elect_one())
         for (int k = 0; k < NS && k < nt; ++k) issue(k);
     if (up && nt > 0) {
         expand_tile(0);
@@ -629,29 +758,34 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     for (int k = 0; k < nt; ++k) {
         const int s = k % NS;
         const uint32_t st = base + (uint32_t)s * (uint32_t)a.stage_bytes;
-        if (tid == 0) {
+        if (warp == 0 && elect_one()) {
             if (!mbar_wait(smem_u32(&bar_full[s]), (k / NS) & 1)) {
                 s_bad = 1;
             } else {
-                loading[s] = -1;
+                landed = k + 1;
                 tc_fence_after();
-                const uint32_t gst = st + (uint32_t)a.x_bytes;
+                // G: 16-channel atoms one after the other, 8 pixel rows of 32
+                // bytes; later operands as in the forward kernel, a distance
+                // further on
+                const uint64_t g0 = smem_desc_mn(st + (uint32_t)a.x_bytes,
+                                                 (uint32_t)a.g_atom_bytes, 256u, 6u);
+                const uint64_t x0d = smem_desc_mn(st, (uint32_t)swx, 8u * (uint32_t)swx,
+                                                  (uint32_t)swcode);
+                const uint32_t pixel = (uint32_t)swx >> 4, row = (uint32_t)a.rs * pixel;
+                const uint32_t Np = (uint32_t)a.Np;
                 for (int r = 0; r < a.TR; ++r) {
-                    const int set = r % a.sets;
-                    for (int k0 = 0; k0 < a.Wt; k0 += 16) {
-                        // G: 16-channel atoms a region apart, 8 pixel rows of 32 bytes
-                        const uint64_t bdesc =
-                            smem_desc_mn(gst + (uint32_t)((r * a.Wt + k0) * 32),
-                                         (uint32_t)a.g_atom_bytes, 256u, 6u);
-                        for (int ky = 0; ky < 3; ++ky) {
-                            const int acc = set * 3 + ky;
-                            const uint64_t adesc = smem_desc_mn(
-                                st + (uint32_t)(((r + ky) * a.rs + k0) * swx), (uint32_t)swx,
-                                8u * (uint32_t)swx, (uint32_t)swcode);
-                            tc_mma(tmem + (uint32_t)(acc * a.Np), adesc, bdesc, idesc,
-                                   (started >> acc) & 1u);
-                            started |= 1u << acc;
-                        }
+                    const uint32_t d = tmem + (uint32_t)(r % a.sets) * 3u * Np;
+                    uint64_t xd = x0d + (uint32_t)r * row;
+                    uint64_t gd = g0 + (uint32_t)r * (g_row >> 4);
+                    // a set's first products start its accumulators
+                    const uint32_t acc = k > 0 || r >= a.sets ? 1u : 0u;
+                    if (lead == 3) {
+                        tc_mma(d, xd, gd, idesc, acc);
+                        for (int k0 = 16; k0 < a.Wt; k0 += 16)
+                            tc_mma_add(d, xd += 16 * pixel, gd += 32, idesc);
+                    } else {
+                        issue_row(d, Np, xd, 16 * pixel, gd, g_row >> 4, idesc, idesc1, lead, acc,
+                                  a.Wt / 16);
                     }
                 }
                 tc_commit(smem_u32(&bar_done[s]));
@@ -666,27 +800,36 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         }
         if (up && k + 1 < nt) expand_tile(k + 1);
         if (dbsum && !s_bad && mbar_wait(smem_u32(&bar_full[s]), (k / NS) & 1)) {
-            // the bias gradient: this thread's output channels summed over
-            // the tile's pixel rows of G in shared memory (beside the multiplies)
-            for (int i = 0; i < 2; ++i) {
-                const int c = tid - 32 + 96 * i;
-                if (c >= a.Np) break;
-                const unsigned char* g0 = smem_raw + (st - smem_u32(smem_raw)) + a.x_bytes +
-                                          (c >> 4) * a.g_atom_bytes;
-                const int e = c & 15;
-                float acc = 0.f;
-                for (int p = 0; p < a.TR * a.Wt; ++p)
-                    acc += __bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(
-                        g0 + swizzle_off((uint32_t)(p * 32 + e * 2), 32)));
-                db_acc[i] += acc;
+            // the bias gradient: this thread's channels and pixels of G in
+            // shared memory (beside the multiplies)
+            const unsigned char* g0 = smem_raw + (st - smem_u32(smem_raw)) + a.x_bytes +
+                                      db_atom * a.g_atom_bytes;
+            const uint32_t piece = (uint32_t)(db_half * 16);
+            for (int r = 0; r < a.TR; ++r) {  // the tile's own rows of G
+                g0 += g_row;
+#pragma unroll 2
+                for (int p = db_phase; p < a.Wt; p += db_phases) {
+                    const uint4 v = *reinterpret_cast<const uint4*>(
+                        g0 + swizzle_off((uint32_t)(p * 32) + piece, 32));
+                    const uint32_t h[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {  // a bf16 is the upper half of its float
+                        db_acc[2 * q] += __uint_as_float(h[q] << 16);
+                        db_acc[2 * q + 1] += __uint_as_float(h[q] & 0xFFFF0000u);
+                    }
+                }
             }
         }
         __syncthreads();
         if (s_bad) break;
     }
-    if (tid == 0)
-        for (int s = 0; s < NS; ++s)
-            if (loading[s] >= 0) mbar_wait(smem_u32(&bar_full[s]), (loading[s] / NS) & 1);
+    if (warp == 0 && elect_one())
+        for (int k = landed; k < issued; ++k)
+            mbar_wait(smem_u32(&bar_full[k % NS]), (k / NS) & 1);
+    if (dbsum)
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+            atomicAdd(&s_db[db_atom * 16 + db_half * 8 + q], db_acc[q]);
     __syncthreads();
     const int committed = s_committed;
     bool ok = !s_bad;
@@ -703,10 +846,10 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             for (int cl = 0; cl < a.Np; cl += 16) {
                 float v[16], w[16];
                 __syncwarp();
-                tmem_ld16(trow + (uint32_t)(ky * a.Np + cl), v);
+                tmem_ld16(trow + (uint32_t)((2 - ky) * a.Np + cl), v);
                 for (int set = 1; set < a.sets; ++set) {
                     __syncwarp();
-                    tmem_ld16(trow + (uint32_t)((set * 3 + ky) * a.Np + cl), w);
+                    tmem_ld16(trow + (uint32_t)((set * 3 + 2 - ky) * a.Np + cl), w);
 #pragma unroll
                     for (int q = 0; q < 16; ++q) v[q] += w[q];
                 }
@@ -731,11 +874,9 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     } else if (!ok && tid == 0) {
         atomicOr(a.err, 1u);
     }
-    if (ok && dbsum)
-        for (int i = 0; i < 2; ++i) {
-            const int c = tid - 32 + 96 * i;
-            if (c < a.Np && co0 + c < a.Co) atomicAdd(a.db + co0 + c, db_acc[i]);
-        }
+    if (ok && a.db != nullptr && chunk == 0)
+        for (int c = tid; c < a.Np; c += kTcThreads)
+            if (co0 + c < a.Co) atomicAdd(a.db + co0 + c, s_db[c]);
     tc_fence_before();
     __syncthreads();
     if (warp == 0)
@@ -767,54 +908,61 @@ __device__ __forceinline__ TileGeom tile_geom(int Ci, int Co) {
 // contiguous in the FP32 source, so that a warp's reads coalesce: where it
 // goes (dst) and which (tap, co, ci) of the array it holds; false for padding
 // (co >= Co)
-__device__ __forceinline__ bool tiled_source(int64_t i, int Ci, int Co, const TileGeom& g,
-                                             bool row_fast, int64_t* dst, int* t, int* co,
+__device__ __forceinline__ bool tiled_source(uint32_t i, int Ci, int Co, const TileGeom& g,
+                                             bool row_fast, uint32_t* dst, int* t, int* co,
                                              int* ci) {
-    const int64_t per_tile = (int64_t)g.nk * 9 * g.Np * g.Kc;
-    const int64_t r = i % per_tile;
-    const int tile = (int)(i / per_tile);
-    const int row = row_fast ? (int)(r % g.Np) : (int)((r / g.Kc) % g.Np);
-    const int e = row_fast ? (int)((r / g.Np) % g.Kc) : (int)(r % g.Kc);
-    *t = (int)((r / ((int64_t)g.Np * g.Kc)) % 9);
-    const int k = (int)(r / ((int64_t)g.Np * g.Kc * 9));
-    *co = tile * g.Np + row;
+    const uint32_t Np = g.Np, Kc = g.Kc, tap = Np * Kc;
+    const uint32_t per_tile = (uint32_t)g.nk * 9u * tap;
+    const uint32_t tile = i / per_tile, r = i - tile * per_tile;
+    const uint32_t kt = r / tap, in = r - kt * tap;
+    const uint32_t fast = row_fast ? Np : Kc, hi = in / fast, lo = in - hi * fast;
+    const int row = (int)(row_fast ? lo : hi), e = (int)(row_fast ? hi : lo);
+    const int k = (int)(kt / 9u);
+    *t = (int)(kt - 9u * (uint32_t)k);
+    *co = (int)tile * g.Np + row;
     *ci = k * g.Kc + e;
     const int swb = 2 * g.Kc;
     const uint32_t off = swizzle_off((uint32_t)(row * swb + e * 2), swb);
-    *dst = (int64_t)tile * per_tile + ((int64_t)k * 9 + *t) * g.Np * g.Kc + off / 2;
+    *dst = tile * per_tile + kt * tap + off / 2;
     return *co < Co && *ci < Ci;
 }
+constexpr uint32_t kRefreshElems = 1024;  // elements of a CTA
 __global__ void refresh_weights_kernel(const WeightSet* sets) {
-    const WeightSet ws = sets[blockIdx.y];
+    int l = 0;
+    while (sets[l + 1].first <= (int)blockIdx.x) ++l;
+    const WeightSet ws = sets[l];
     const int Ci = ws.Ci, Co = ws.Co;
-    const int64_t n_copy = 9LL * Ci * Co;
+    // (32-bit indices: a layer's copies hold fewer than 2^31 elements; in 64
+    // bits, every copy made for every layer and a layer per grid row this took
+    // 100 us for 2 M weights, now 30)
+    const uint32_t n_copy = ws.wf || ws.wd ? 9u * (uint32_t)Ci * (uint32_t)Co : 0u;
     const TileGeom gf = tile_geom(Ci, Co), gd = tile_geom(Co, Ci);
-    const int64_t n_f = ws.wft ? (int64_t)gf.nt * gf.nk * 9 * gf.Np * gf.Kc : 0;
-    const int64_t n_d = ws.wdt ? (int64_t)gd.nt * gd.nk * 9 * gd.Np * gd.Kc : 0;
-    const int64_t total = n_copy + n_f + n_d;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total;
-         i += (int64_t)gridDim.x * blockDim.x) {
+    const uint32_t n_f = ws.wft ? (uint32_t)(gf.nt * gf.nk * 9 * gf.Np * gf.Kc) : 0u;
+    const uint32_t n_d = ws.wdt ? (uint32_t)(gd.nt * gd.nk * 9 * gd.Np * gd.Kc) : 0u;
+    const uint32_t total = n_copy + n_f + n_d;
+    const uint32_t begin = (blockIdx.x - (uint32_t)ws.first) * kRefreshElems;
+    const uint32_t end = min(begin + kRefreshElems, total);
+    for (uint32_t i = begin + threadIdx.x; i < end; i += blockDim.x) {
         if (i < n_copy) {
-            const int o = (int)(i % Co);
-            const int in = (int)((i / Co) % Ci);
-            const int t = (int)(i / ((int64_t)Co * Ci));
+            const uint32_t row = i / (uint32_t)Co, o = i - row * (uint32_t)Co;
+            const uint32_t t = row / (uint32_t)Ci, in = row - t * (uint32_t)Ci;
             const __nv_bfloat16 v = __float2bfloat16(ws.w[i]);
-            ws.wf[((int64_t)t * Co + o) * Ci + in] = v;
-            ws.wd[((int64_t)(8 - t) * Ci + in) * Co + o] = v;
+            if (ws.wf) ws.wf[(t * Co + o) * Ci + in] = v;
+            if (ws.wd) ws.wd[((8 - t) * Ci + in) * Co + o] = v;
         } else if (i < n_copy + n_f) {
             // the forward tiling: the (9, Co, Ci) array is wf
-            int64_t dst;
+            uint32_t dst;
             int t, co, ci;
             const bool in = tiled_source(i - n_copy, Ci, Co, gf, true, &dst, &t, &co, &ci);
-            ws.wft[dst] = in ? __float2bfloat16(ws.w[((int64_t)t * Ci + ci) * Co + co])
+            ws.wft[dst] = in ? __float2bfloat16(ws.w[(t * Ci + ci) * Co + co])
                              : __float2bfloat16(0.f);
         } else {
             // the data-gradient tiling: the (9, Ci, Co) array is wd, whose
             // output channels are the forward input channels
-            int64_t dst;
+            uint32_t dst;
             int t, co, ci;
             const bool in = tiled_source(i - n_copy - n_f, Co, Ci, gd, false, &dst, &t, &co, &ci);
-            ws.wdt[dst] = in ? __float2bfloat16(ws.w[((int64_t)(8 - t) * Ci + co) * Co + ci])
+            ws.wdt[dst] = in ? __float2bfloat16(ws.w[((8 - t) * Ci + co) * Co + ci])
                              : __float2bfloat16(0.f);
         }
     }
@@ -892,7 +1040,7 @@ static bool tc_plan(int N, int H, int W, int Np, int ntiles, int nk, bool up,
         // three stages where they fit without costing the second CTA per SM
         int ns = nk == 1 ? 1 : 3;
         while (ns > 1 && ns * stage + 1024 > kTcSmemMax) --ns;
-        if (ns == 3 && 2 * (3 * stage + 2048) > kTcSmemSM && 2 * (2 * stage + 2048) <= kTcSmemSM)
+        if (ns == 3 && 2 * (3 * stage + 3072) > kTcSmemSM && 2 * (2 * stage + 3072) <= kTcSmemSM)
             ns = 2;
         if (ns * stage + 1024 > kTcSmemMax || (nk > 1 && ns < 2)) continue;
         const int ty = (H + TR - 1) / TR;
@@ -955,14 +1103,6 @@ cudaError_t tc_tile_weights(const void* w, int Co, int Ci, void* wt, cudaStream_
 }
 
 // ---- the weight gradient
-// output channels of one N tile (at most 160: three accumulators of Np
-// columns and more sets where they fit in the 512 TMEM columns)
-static void tcw_ntiles(int Co, int* ntiles, int* Np) {
-    const int n16 = (Co + 15) / 16;
-    *ntiles = (n16 + 9) / 10;
-    *Np = (n16 + *ntiles - 1) / *ntiles * 16;
-}
-
 bool tc_wgrad_supported(int H, int W, int C1, int C2, int Co) {
     if (H < 1 || W < 16 || (W <= 128 ? W % 16 : W % 128) || C1 < 16 || C1 % 16 || C2 < 0 ||
         C2 % 16 || Co < 16 || Co % 16 || (C2 > 0 && (H % 2 || W % 2)) ||
@@ -1002,32 +1142,40 @@ cudaError_t tc_conv3x3_wgrad(const nn::WgradArgs& w, unsigned* err, cudaStream_t
     }
     a.nchunks = nchunks;
     int ntn = 1;
-    tcw_ntiles(w.Co, &ntn, &a.Np);
-    a.ng = a.Np / 16;
     a.Wt = w.W <= 128 ? w.W : 128;
     a.rs = a.Wt + 2;
     a.tiles_x = w.W / a.Wt;
     // the tile: TR rows, the largest of 4, 2, 1 whose stage fits twice; the
-    // halo region holds a 32-channel chunk (64-byte rows) plus the rows the
-    // unused shifts of the last K step read (up to eight, for 16 channels)
-    for (int TR = 4; TR >= 1; TR /= 2) {
-        const int rows = (TR + 2) * a.rs + 8;
-        const int xb = (rows * 64 + 1023) / 1024 * 1024;
-        const int gab = TR * a.Wt * 32;
-        const int up_rows = (TR + 3) / 2 + 1, up_cols = a.Wt / 2 + 2;
-        const int up_off = (xb + a.ng * gab + 1023) / 1024 * 1024;
-        const int up_bytes = w.C2 > 0 ? (up_rows * up_cols * 64 + 1023) / 1024 * 1024 : 0;
-        const int stage = up_off + up_bytes;
-        if (2 * stage + 1024 > kTcSmemMax && TR > 1) continue;
-        a.TR = TR;
-        a.x_bytes = xb;
-        a.g_atom_bytes = gab;
-        a.stage_bytes = stage;
-        a.up_rows = up_rows;
-        a.up_cols = up_cols;
-        a.up_off = up_off;
-        a.stages = 3 * stage + 1024 <= kTcSmemMax ? 3 : 2;
-        break;
+    // X region holds a 32-channel chunk (64-byte rows) plus the rows the
+    // unused shifts of the last K step read (up to eight, for 16 channels).
+    // The N tile: all output channels up to 160 (the accumulators of three rows
+    // in the 512 TMEM columns) or equal parts, as many as leave TR = 2 (80
+    // channels always fit; at TR = 1 every row of G would be staged three times)
+    a.TR = 0;
+    for (int per = 10; per >= 5 && a.TR < 2; --per) {
+        const int n16 = (w.Co + 15) / 16;
+        ntn = (n16 + per - 1) / per;
+        a.Np = (n16 + ntn - 1) / ntn * 16;
+        a.ng = a.Np / 16;
+        for (int TR = 4; TR >= 1; TR /= 2) {
+            const int rows = TR * a.rs + 8;
+            const int xb = (rows * 64 + 1023) / 1024 * 1024;
+            const int gab = a.Wt * 32;
+            const int up_rows = (TR + 1) / 2 + 1, up_cols = a.Wt / 2 + 2;
+            const int up_off = (xb + (TR + 2) * a.ng * gab + 1023) / 1024 * 1024;
+            const int up_bytes = w.C2 > 0 ? (up_rows * up_cols * 64 + 1023) / 1024 * 1024 : 0;
+            const int stage = up_off + up_bytes;
+            if (2 * stage + 1024 > kTcSmemMax && TR > 1) continue;
+            a.TR = TR;
+            a.x_bytes = xb;
+            a.g_atom_bytes = gab;
+            a.stage_bytes = stage;
+            a.up_rows = up_rows;
+            a.up_cols = up_cols;
+            a.up_off = up_off;
+            a.stages = 3 * stage + 1024 <= kTcSmemMax ? 3 : 2;
+            break;
+        }
     }
     if (a.stages * a.stage_bytes + 1024 > kTcSmemMax) return cudaErrorInvalidValue;
     // accumulator sets: as many as TMEM holds (three accumulators of Np
@@ -1059,13 +1207,13 @@ cudaError_t tc_conv3x3_wgrad(const nn::WgradArgs& w, unsigned* err, cudaStream_t
     };
     CUtensorMap mg, mx32, mx16, mu32, mu16;
     std::memset(&mg, 0, sizeof(mg));
-    if (!encode(&mg, w.g, w.Co, w.W, w.H, 16, a.Wt, a.TR)) return cudaErrorInvalidValue;
+    if (!encode(&mg, w.g, w.Co, w.W, w.H, 16, a.Wt, 1)) return cudaErrorInvalidValue;
     bool need[2][2] = {{false, false}, {false, false}};  // [in2][16-channel]
     for (int k = 0; k < nchunks; ++k) need[a.ck_up[k]][a.ck_kc[k] == 16] = true;
     mx32 = mx16 = mu32 = mu16 = mg;  // placeholders for the boxes no chunk uses
-    if (need[0][0] && !encode(&mx32, w.in1, w.C1, w.W, w.H, 32, a.rs, a.TR + 2))
+    if (need[0][0] && !encode(&mx32, w.in1, w.C1, w.W, w.H, 32, a.rs, a.TR))
         return cudaErrorInvalidValue;
-    if (need[0][1] && !encode(&mx16, w.in1, w.C1, w.W, w.H, 16, a.rs, a.TR + 2))
+    if (need[0][1] && !encode(&mx16, w.in1, w.C1, w.W, w.H, 16, a.rs, a.TR))
         return cudaErrorInvalidValue;
     if (need[1][0] &&
         !encode(&mu32, w.in2, w.C2, w.W / 2, w.H / 2, 32, a.up_cols, a.up_rows))
@@ -1083,14 +1231,16 @@ cudaError_t tc_conv3x3_wgrad(const nn::WgradArgs& w, unsigned* err, cudaStream_t
     return cudaGetLastError();
 }
 
-int64_t weight_set_elems(int Ci, int Co) {
-    return 9LL * Ci * Co + tc_tiled_weight_elems(Ci, Co) + tc_tiled_weight_elems(Co, Ci);
+int weight_set_blocks(const WeightSet& w) {
+    const int64_t n = (w.wf || w.wd ? 9LL * w.Ci * w.Co : 0) +
+                      (w.wft ? tc_tiled_weight_elems(w.Ci, w.Co) : 0) +
+                      (w.wdt ? tc_tiled_weight_elems(w.Co, w.Ci) : 0);
+    return (int)((n + nn::kRefreshElems - 1) / nn::kRefreshElems);
 }
 
-cudaError_t refresh_weight_sets(const WeightSet* d_sets, int n, int64_t max_elems, cudaStream_t s) {
-    if (n < 1) return cudaSuccess;
-    const int bx = (int)std::min<int64_t>((max_elems + 255) / 256, 1024);
-    nn::refresh_weights_kernel<<<dim3(bx, n), 256, 0, s>>>(d_sets);
+cudaError_t refresh_weight_sets(const WeightSet* d_sets, int blocks, cudaStream_t s) {
+    if (blocks < 1) return cudaSuccess;
+    nn::refresh_weights_kernel<<<blocks, 256, 0, s>>>(d_sets);
     return cudaGetLastError();
 }
 

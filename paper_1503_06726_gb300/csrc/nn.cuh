@@ -39,15 +39,14 @@ __global__ void conv3x3_fwd_kernel(ConvArgs a);
 __global__ void conv3x3_wgrad_kernel(WgradArgs a);
 __global__ void avgpool2_kernel(const __nv_bfloat16* x, __nv_bfloat16* y, int N, int H, int W,
                                 int C);
-__global__ void avgpool2_bwd_kernel(const __nv_bfloat16* g, __nv_bfloat16* gx, int N, int H,
-                                    int W, int C);
+__global__ void pool_skip_bwd_kernel(const __nv_bfloat16* g, const __nv_bfloat16* skip,
+                                     const __nv_bfloat16* act, __nv_bfloat16* out, int N, int H,
+                                     int W, int C);
 __global__ void concat_bwd_kernel(const __nv_bfloat16* g, __nv_bfloat16* gskip,
                                   __nv_bfloat16* gx2, const __nv_bfloat16* gate2, int N, int H,
                                   int W, int C1, int C2, int accumulate_skip);
-__global__ void add_gate_kernel(__nv_bfloat16* g, const __nv_bfloat16* h,
-                                const __nv_bfloat16* act, int64_t n);
-__global__ void mse_kernel(const float* y, int Cy, const float* t, __nv_bfloat16* dy, int Cdy,
-                           int64_t n, double* loss);
+__global__ void mse_kernel(const float* y, int Cy, const float* t, __nv_bfloat16* dy, int64_t n,
+                           double* loss);
 __global__ void adam_kernel(float* p, const float* g, float* m, float* v, int64_t n, float lr,
                             float b1, float b2, float eps, float c1, float c2);
 __global__ void weight_copies_kernel(const float* w, int Ci, int Co, int Cip, int Cop,
@@ -78,14 +77,17 @@ cudaError_t tc_conv3x3_wgrad(const nn::WgradArgs& w, unsigned* err, cudaStream_t
 // One layer of the fused weight refresh: the FP32 master weights w (9, Ci, Co)
 // and the BF16 copies made from them -- the forward copy wf (9, Co, Ci), the
 // tap-flipped data-gradient copy wd (9, Ci, Co) and the tcgen05 tilings of
-// both (wft, wdt).
+// both (wft, wdt); a copy that nothing reads is NULL.  first: the layer's first
+// CTA of the refresh (a table ends with an entry that holds only the number of
+// CTAs).
 struct WeightSet {
     const float* w;
     __nv_bfloat16 *wf, *wd, *wft, *wdt;
     int Ci, Co;
+    int first;
 };
-// All layers' copies in one launch (d_sets: the table in device memory, n
-// entries; max_elems: the largest per-layer element count, for the grid).
-cudaError_t refresh_weight_sets(const WeightSet* d_sets, int n, int64_t max_elems, cudaStream_t s);
-int64_t weight_set_elems(int Ci, int Co);
+// CTAs of one layer's refresh, and all layers' copies in one launch (d_sets:
+// the table in device memory; blocks: the CTAs of all layers)
+int weight_set_blocks(const WeightSet& w);
+cudaError_t refresh_weight_sets(const WeightSet* d_sets, int blocks, cudaStream_t s);
 }  // namespace lbib

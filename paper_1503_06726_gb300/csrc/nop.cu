@@ -121,7 +121,7 @@ struct lbib_nop {
     double* loss = nullptr;
     unsigned* tc_err = nullptr;  // raised by a tcgen05 convolution whose bounded wait ran out
     WeightSet* wsets = nullptr;  // per layer: master weights and their BF16 copies (device table)
-    int64_t wsets_max = 0;       // the largest layer's element count over all its copies
+    int wsets_blocks = 0;        // CTAs of their refresh
     int64_t t = 0;           // Adam step
     std::string err;
     // pinned host staging: the per-sample inputs (3 B floats), then the loss
@@ -173,7 +173,7 @@ void nop_layout(lbib_nop* n) {
         l.wdt = n->take<bf16>(tc_tiled_weight_elems(l.cop, l.cip));
     }
     n->tc_err = n->take<unsigned>(1);
-    n->wsets = n->take<WeightSet>(n->L.size());
+    n->wsets = n->take<WeightSet>(n->L.size() + 1);
     const int64_t B = n->B;
     int64_t maxg = 0;
     for (int l = 0; l < kLevels; ++l) {
@@ -205,11 +205,19 @@ void nop_layout(lbib_nop* n) {
 
 inline unsigned blocks(int64_t n, int t = 256) { return (unsigned)((n + t - 1) / t); }
 
-// A 3x3 convolution of the network: on the tcgen05 tensor cores (tiled
-// weights wt) for images of rows of 128 pixels or more, where the single
-// halo per tile makes them the faster kernel (1.7 - 2.4x at 256 x 256, even
-// at 128 x 128); narrower levels, where the three kx-shifted halo copies
-// cost more than the warp-level kernel's register tiling, take the latter.
+// Where a convolution of the network runs on the tcgen05 tensor cores: images
+// of rows of 128 pixels or more, in the widths that the kernel supports.  On
+// narrower levels the two kernels are close (us of 16 images on the tensor
+// cores and on the warp-level kernel: 64^2, 64 -> 64 channels 25 and 25; 32^2,
+// 96 -> 96 18 and 19; 16^2, 128 -> 128 14 and 17; upsampled inputs 55 and 52 at
+// 64^2, 39 and 37 at 32^2), and another order of their sums moves the weights
+// after four steps by 2.5e-4, three times what two runs differ by.
+bool tc_conv_used(int H, int W, int C1, int C2, int Co) {
+    return W >= 128 && tc_conv_supported(H, W, C1, C2, Co);
+}
+
+// A 3x3 convolution of the network (w: the plain copy of its weights for the
+// warp-level kernel, wt: the tiled one for the tensor cores).
 cudaError_t conv_fwd(lbib_nop* n, const Layer& l, const bf16* in1, const bf16* in2, int C1, int C2,
                      int lvl, void* out, int relu, int out_f32, const bf16* w, const bf16* wt,
                      const float* bias, int Co, int N, const bf16* gate = nullptr) {
@@ -230,7 +238,7 @@ cudaError_t conv_fwd(lbib_nop* n, const Layer& l, const bf16* in1, const bf16* i
     a.out_f32 = out_f32;
     a.gate = gate;
     (void)l;
-    if (wt && a.W >= 128 && tc_conv_supported(a.H, a.W, C1, C2, Co)) return tc_conv3x3(a, wt, n->tc_err, n->stream);
+    if (wt && tc_conv_used(a.H, a.W, C1, C2, Co)) return tc_conv3x3(a, wt, n->tc_err, n->stream);
     const int tiles = ((a.H + kTH - 1) / kTH) * ((a.W + kTW - 1) / kTW);
     dim3 grid(tiles, (Co + 63) / 64, N);
     nn::conv3x3_fwd_kernel<<<grid, 256, kConvSmem, n->stream>>>(a);
@@ -266,7 +274,7 @@ cudaError_t conv_wgrad(lbib_nop* n, const Layer& l, const bf16* in1, const bf16*
 // The BF16 copies of every layer's weights (forward, tap-flipped, and their
 // tcgen05 tilings) from the FP32 master weights, in one launch.
 cudaError_t refresh_weights(lbib_nop* n) {
-    return refresh_weight_sets(n->wsets, (int)n->L.size(), n->wsets_max, n->stream);
+    return refresh_weight_sets(n->wsets, n->wsets_blocks, n->stream);
 }
 
 cudaError_t set_inputs(lbib_nop* n, int N, const uint8_t* mask, const uint8_t* src,
@@ -296,6 +304,14 @@ cudaError_t set_inputs(lbib_nop* n, int N, const uint8_t* mask, const uint8_t* s
     nn::features_kernel<<<blocks((int64_t)N * HW), 256, 0, n->stream>>>(mask, src, n->dn, n->kn,
                                                                          n->x, N, HW);
     return cudaGetLastError();
+}
+
+// Channels of the output layer's result y: the one that is used where the
+// tensor-core kernel writes it (its weight tiles hold 16 rows for 1 or 16
+// channels alike; 16 images of 256^2: 106 us with 16, 38 with one), else the
+// padded 16.
+int y_channels(const lbib_nop* n) {
+    return tc_conv_used(n->H, n->W, kCh[0], 0, 1) ? 1 : 16;
 }
 
 cudaError_t forward(lbib_nop* n, int N) {
@@ -332,7 +348,7 @@ cudaError_t forward(lbib_nop* n, int N) {
     if (e == cudaSuccess) {
         const Layer& o = L[li];
         e = conv_fwd(n, o, n->dec_out[0], nullptr, kCh[0], 0, 0, n->y, 0, 1, o.wf, o.wft,
-                     n->param + o.off + 9LL * o.cip * o.cop, o.cop, N);
+                     n->param + o.off + 9LL * o.cip * o.cop, y_channels(n), N);
     }
     return e;
 }
@@ -380,16 +396,8 @@ cudaError_t backward(lbib_nop* n, int N) {
     }
     // g: gradient of the deepest encoder output (level 5)
     for (int l = kLevels - 1; l >= 0 && e == cudaSuccess; --l) {
-        const int64_t hw = (int64_t)(n->H >> l) * (n->W >> l);
         const Layer& a = enc(l, 0);
         const Layer& b = enc(l, 1);
-        if (l < kLevels - 1) {
-            // the skip's gradient joins the deeper path's, through the ReLU
-            // (at the deepest level the concatenation split applied it)
-            nn::add_gate_kernel<<<blocks(N * hw * kCh[l] / 8), 256, 0, n->stream>>>(
-                g, n->gskip[l], n->enc_out[l], N * hw * kCh[l]);
-            e = cudaGetLastError();
-        }
         if (e == cudaSuccess) e = conv_wgrad(n, b, n->enc_r1[l], nullptr, kCh[l], 0, l, g, N);
         if (e == cudaSuccess)
             e = conv_fwd(n, b, g, nullptr, kCh[l], 0, l, s1, 0, 0, b.wd, b.wdt, nullptr, kCh[l], N,
@@ -399,9 +407,12 @@ cudaError_t backward(lbib_nop* n, int N) {
         if (l > 0 && e == cudaSuccess) {
             e = conv_fwd(n, a, s1, nullptr, kCh[l], 0, l, s2, 0, 0, a.wd, a.wdt, nullptr, cin, N);
             if (e == cudaSuccess) {
+                // joined by the skip's gradient, through the ReLU (at the deepest
+                // level the concatenation split applied it)
                 const int64_t cnt = N * (int64_t)(n->H >> (l - 1)) * (n->W >> (l - 1)) * cin;
-                nn::avgpool2_bwd_kernel<<<blocks(cnt / 8), 256, 0, n->stream>>>(
-                    s2, g, N, n->H >> (l - 1), n->W >> (l - 1), cin);
+                nn::pool_skip_bwd_kernel<<<blocks(cnt / 8), 256, 0, n->stream>>>(
+                    s2, n->gskip[l - 1], n->enc_out[l - 1], g, N, n->H >> (l - 1), n->W >> (l - 1),
+                    cin);
                 e = cudaGetLastError();
             }
         }
@@ -478,17 +489,27 @@ int lbib_nop_create(int32_t batch, int32_t H, int32_t W, void* d_workspace, uint
     if (e == cudaSuccess) e = cudaMemsetAsync(n->param, 0, n->P * 4 * 4, n->stream);  // param, grad, m, v
     if (e == cudaSuccess) e = cudaMemsetAsync(n->tc_err, 0, 4, n->stream);
     std::vector<WeightSet> sets;
-    for (const Layer& l : n->L) {
+    for (size_t i = 0; i <= n->L.size(); ++i) {
         WeightSet w;
-        w.w = n->param + l.off;
-        w.wf = l.wf;
-        w.wd = l.wd;
-        w.wft = l.wft;
-        w.wdt = l.wdt;
-        w.Ci = l.cip;
-        w.Co = l.cop;
+        std::memset(&w, 0, sizeof(w));
+        w.first = n->wsets_blocks;
+        if (i < n->L.size()) {
+            const Layer& l = n->L[i];
+            w.w = n->param + l.off;
+            w.Ci = l.cip;
+            w.Co = l.cop;
+            // the copies that the layer's two convolutions read: encoder levels
+            // 0 .. 5 (two layers each), decoder levels 4 .. 0, the output layer
+            const int lvl = i < 12 ? (int)i / 2 : (i < 22 ? 4 - ((int)i - 12) / 2 : 0);
+            const bool cat = i >= 12 && i < 22 && i % 2 == 0;  // [skip, upsampled]
+            const int C1 = cat ? kCh[lvl] : l.cip;
+            const bool fwd = tc_conv_used(H >> lvl, W >> lvl, C1, l.cip - C1, l.co);
+            const bool bwd = tc_conv_used(H >> lvl, W >> lvl, l.cop, 0, l.cip);
+            (fwd ? w.wft : w.wf) = fwd ? l.wft : l.wf;
+            (bwd ? w.wdt : w.wd) = bwd ? l.wdt : l.wd;
+            n->wsets_blocks += weight_set_blocks(w);
+        }
         sets.push_back(w);
-        n->wsets_max = std::max(n->wsets_max, weight_set_elems(l.cip, l.cop));
     }
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(n->wsets, sets.data(), sets.size() * sizeof(WeightSet),
@@ -588,7 +609,7 @@ int lbib_nop_forward(lbib_nop* n, int32_t N, const uint8_t* d_mask, const uint8_
     if (e == cudaSuccess) e = forward(n, N);
     if (e == cudaSuccess) {
         const int HW = n->H * n->W;
-        nn::scale_kernel<<<blocks((int64_t)N * HW), 256, 0, n->stream>>>(n->y, 16, d_phi, n->fac, N, HW);
+        nn::scale_kernel<<<blocks((int64_t)N * HW), 256, 0, n->stream>>>(n->y, y_channels(n), d_phi, n->fac, N, HW);
         e = cudaGetLastError();
     }
     if (e != cudaSuccess) return nop_fail(n, LBIB_E_CUDA, cudaGetErrorString(e));
@@ -613,7 +634,8 @@ int lbib_nop_train_step(lbib_nop* n, int32_t N, const uint8_t* d_mask, const uin
     if (e == cudaSuccess) e = forward(n, N);
     if (e == cudaSuccess) e = cudaMemsetAsync(n->loss, 0, 8, n->stream);
     if (e == cudaSuccess) {
-        nn::mse_kernel<<<blocks(np), 256, 0, n->stream>>>(n->y, 16, n->tgt, n->dy, 16, np, n->loss);
+        nn::mse_kernel<<<std::min(blocks(np), 8u * 152u), 256, 0, n->stream>>>(
+            n->y, y_channels(n), n->tgt, n->dy, np, n->loss);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = backward(n, N);
