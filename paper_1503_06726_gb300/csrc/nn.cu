@@ -47,13 +47,20 @@ constexpr int HH = TH + 2, HWD = TW + 2;   // halo tile
 constexpr int AST = KC + 8;                // smem row stride (bf16) of halo / weight rows
 constexpr int kConvThreads = 256;
 constexpr int kHaloBytes = HH * HWD * AST * 2;
-constexpr int kWBytes = 9 * BN * AST * 2;
-static_assert(kConvSmem == kHaloBytes + kWBytes, "conv smem");
+constexpr int kFewCtas = 152;
 
 __device__ __forceinline__ void cp_async16(void* smem, const void* gmem, bool valid) {
     const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
     const int n = valid ? 16 : 0;
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(s), "l"(gmem), "r"(n));
+}
+__device__ __forceinline__ void cp_async_commit() {
+    asm volatile("cp.async.commit_group;\n" ::);
+}
+// until at most N of the committed groups are in flight
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+    asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
 }
 __device__ __forceinline__ void cp_async_wait_all() {
     asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;\n" ::);
@@ -102,10 +109,22 @@ __device__ __forceinline__ void load_halo(const ConvArgs& a, int n, int y0, int 
     }
 }
 
-__global__ void __launch_bounds__(kConvThreads) conv3x3_fwd_kernel(ConvArgs a) {
+// WN: warps along the output channels (32 each), STAGES: chunks of operands
+// whose copies are in flight or in use.  {2, 1}: 60 KB, three CTAs per SM hide
+// each other's copies (held to 85 registers for the third).  {1, 3}: where the
+// grid of the former would leave no SM a second CTA, half the weights per CTA
+// and two chunks ahead.  With few warps per SM the taps are a chain of ldmatrix
+// and mma latencies: unrolled, the next tap's operands load beside this one's
+// multiplies (9 taps with one warp per scheduler, 3 within the 85 registers).
+// 16 images, us: 8^2, 192 -> 192 channels 23.7 -> 14.7 (18.5 without the
+// unrolling), 16^2, 320 -> 128 37 -> 22.4 (29.1), 64^2, 64 -> 64 25.1 -> 22.9;
+// {1, 3} at 32^2, 96 -> 96, 256 CTAs of the other: 25 against 17.5.  The order of
+// a pixel's sums is the same.
+template <int WN, int STAGES>
+__global__ void __launch_bounds__(128 * WN, WN == 2 ? 3 : 1) conv3x3_fwd_kernel(ConvArgs a) {
+    constexpr int BN = 32 * WN;
+    constexpr int kStage = kHaloBytes + 9 * BN * AST * 2;
     extern __shared__ __align__(16) unsigned char smem[];
-    __nv_bfloat16* halo = reinterpret_cast<__nv_bfloat16*>(smem);
-    __nv_bfloat16* wts = reinterpret_cast<__nv_bfloat16*>(smem + kHaloBytes);
     const int tiles_x = (a.W + TW - 1) / TW;
     const int y0 = (blockIdx.x / tiles_x) * TH, x0 = (blockIdx.x % tiles_x) * TW;
     const int co0 = blockIdx.y * BN, n = blockIdx.z;
@@ -121,9 +140,13 @@ __global__ void __launch_bounds__(kConvThreads) conv3x3_fwd_kernel(ConvArgs a) {
 #pragma unroll
             for (int k = 0; k < 4; ++k) acc[i][j][k] = 0.f;
 
-    for (int ci0 = 0; ci0 < Ci; ci0 += KC) {
+    const int nk = (Ci + KC - 1) / KC;
+    auto load = [&](int k) {
+        __nv_bfloat16* halo = reinterpret_cast<__nv_bfloat16*>(smem + (k % STAGES) * kStage);
+        __nv_bfloat16* wts = halo + kHaloBytes / 2;
+        const int ci0 = k * KC;
         load_halo(a, n, y0, x0, ci0, halo);
-        for (int idx = tid; idx < 9 * BN * (KC / 8); idx += blockDim.x) {
+        for (int idx = tid; idx < 9 * BN * (KC / 8); idx += 128 * WN) {
             const int tap = idx / (BN * (KC / 8)), r = idx % (BN * (KC / 8));
             const int co = r / (KC / 8), cc = r % (KC / 8);
             const int gco = co0 + co, ci = ci0 + cc * 8;
@@ -131,9 +154,27 @@ __global__ void __launch_bounds__(kConvThreads) conv3x3_fwd_kernel(ConvArgs a) {
             const __nv_bfloat16* src = ok ? a.w + ((int64_t)tap * a.Co + gco) * Ci + ci : a.w;
             cp_async16(wts + (tap * BN + co) * AST + cc * 8, src, ok);
         }
-        cp_async_wait_all();
-        __syncthreads();
-#pragma unroll 1
+    };
+    // (a group per chunk, empty past the last one, so that the counts stay)
+    for (int k = 0; k < STAGES - 1; ++k) {
+        if (k < nk) load(k);
+        cp_async_commit();
+    }
+    for (int k = 0; k < nk; ++k) {
+        if (STAGES == 1) {
+            load(k);
+            cp_async_wait_all();
+            __syncthreads();
+        } else {
+            cp_async_wait<STAGES - 2>();
+            __syncthreads();  // chunk k has landed; every warp is done with chunk k - 1
+            if (k + STAGES - 1 < nk) load(k + STAGES - 1);
+            cp_async_commit();
+        }
+        const __nv_bfloat16* halo =
+            reinterpret_cast<const __nv_bfloat16*>(smem + (k % STAGES) * kStage);
+        const __nv_bfloat16* wts = halo + kHaloBytes / 2;
+#pragma unroll (WN == 2 ? 3 : 9)
         for (int tap = 0; tap < 9; ++tap) {
             const int ky = tap / 3, kx = tap % 3;
 #pragma unroll
@@ -161,7 +202,7 @@ __global__ void __launch_bounds__(kConvThreads) conv3x3_fwd_kernel(ConvArgs a) {
                     for (int nt = 0; nt < 4; ++nt) mma_bf16(acc[mt][nt], af[mt], bf[nt][0], bf[nt][1]);
             }
         }
-        __syncthreads();
+        if (STAGES == 1) __syncthreads();
     }
 
     // epilogue: bias, ReLU, store (pairs of output channels)
@@ -202,6 +243,23 @@ __global__ void __launch_bounds__(kConvThreads) conv3x3_fwd_kernel(ConvArgs a) {
                 }
             }
         }
+}
+
+template <int WN, int STAGES>
+static cudaError_t launch_fwd(const ConvArgs& a, int tiles, cudaStream_t s) {
+    constexpr int smem = STAGES * (kHaloBytes + 9 * 32 * WN * AST * 2);
+    const cudaError_t e = cudaFuncSetAttribute(conv3x3_fwd_kernel<WN, STAGES>,
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    const dim3 grid(tiles, (a.Co + 32 * WN - 1) / (32 * WN), a.N);
+    conv3x3_fwd_kernel<WN, STAGES><<<grid, 128 * WN, smem, s>>>(a);
+    return cudaGetLastError();
+}
+cudaError_t conv3x3_fwd(const ConvArgs& a, cudaStream_t s) {
+    const int tiles = ((a.H + TH - 1) / TH) * ((a.W + TW - 1) / TW);
+    // 152 SMs: at most one CTA of 64 channels each (see above)
+    if ((int64_t)tiles * ((a.Co + 63) / 64) * a.N <= kFewCtas) return launch_fwd<1, 3>(a, tiles, s);
+    return launch_fwd<2, 1>(a, tiles, s);
 }
 
 // ---------------------------------------------------------------------------

@@ -32,10 +32,10 @@ struct WgradArgs {
 };
 
 constexpr int kTH = 8, kTW = 16;  // pixel tile of a CTA
-constexpr int kConvSmem = (10 * 18 * 40 + 9 * 64 * 40) * 2;
 constexpr int kWgSmem = 10 * 18 * 40 * 2 + 128 * 72 * 2;
 
-__global__ void conv3x3_fwd_kernel(ConvArgs a);
+// the warp-level convolution (forward, data gradient)
+cudaError_t conv3x3_fwd(const ConvArgs& a, cudaStream_t s);
 __global__ void conv3x3_wgrad_kernel(WgradArgs a);
 __global__ void avgpool2_kernel(const __nv_bfloat16* x, __nv_bfloat16* y, int N, int H, int W,
                                 int C);

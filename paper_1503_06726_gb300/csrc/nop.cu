@@ -33,7 +33,6 @@ namespace {
 
 constexpr int kLevels = 6;
 constexpr int kCh[kLevels] = {32, 48, 64, 96, 128, 192};
-using nn::kConvSmem;
 using nn::kTH;
 using nn::kTW;
 using nn::kWgSmem;
@@ -239,10 +238,7 @@ cudaError_t conv_fwd(lbib_nop* n, const Layer& l, const bf16* in1, const bf16* i
     a.gate = gate;
     (void)l;
     if (wt && tc_conv_used(a.H, a.W, C1, C2, Co)) return tc_conv3x3(a, wt, n->tc_err, n->stream);
-    const int tiles = ((a.H + kTH - 1) / kTH) * ((a.W + kTW - 1) / kTW);
-    dim3 grid(tiles, (Co + 63) / 64, N);
-    nn::conv3x3_fwd_kernel<<<grid, 256, kConvSmem, n->stream>>>(a);
-    return cudaGetLastError();
+    return nn::conv3x3_fwd(a, n->stream);
 }
 
 cudaError_t conv_wgrad(lbib_nop* n, const Layer& l, const bf16* in1, const bf16* in2, int C1,
@@ -481,9 +477,6 @@ int lbib_nop_create(int32_t batch, int32_t H, int32_t W, void* d_workspace, uint
     cudaError_t e = cudaHostAlloc(reinterpret_cast<void**>(&n->hpin), n->pin_bytes(),
                                   cudaHostAllocDefault);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(nn::conv3x3_fwd_kernel,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, kConvSmem);
-    if (e == cudaSuccess)
         e = cudaFuncSetAttribute(nn::conv3x3_wgrad_kernel,
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, kWgSmem);
     if (e == cudaSuccess) e = cudaMemsetAsync(n->param, 0, n->P * 4 * 4, n->stream);  // param, grad, m, v
@@ -683,13 +676,7 @@ int lbib_nn_conv3x3(int32_t N, int32_t H, int32_t W, int32_t C1, int32_t C2, int
     a.out_f32 = out_f32;
     a.gate = nullptr;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    cudaError_t e = cudaFuncSetAttribute(nn::conv3x3_fwd_kernel,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, kConvSmem);
-    if (e == cudaSuccess) {
-        const int tiles = ((H + kTH - 1) / kTH) * ((W + kTW - 1) / kTW);
-        nn::conv3x3_fwd_kernel<<<dim3(tiles, (Co + 63) / 64, N), 256, kConvSmem, st>>>(a);
-        e = cudaGetLastError();
-    }
+    const cudaError_t e = nn::conv3x3_fwd(a, st);
     if (e != cudaSuccess) return set_thread_error(LBIB_E_CUDA, cudaGetErrorString(e));
     return LBIB_OK;
 }
