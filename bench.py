@@ -214,15 +214,12 @@ def recorded_traffic(workload_name: str, key: str = "dram_bytes_per_launch", sha
     return None
 
 
-def fp64_flops_per_node(n_species: int, forcing: int) -> int:
-    """FP64 operations of the collision of one node as written (add, sub,
-    mul and reciprocal count 1, fma 2): force 2, moments 26, common even
-    part 18, four direction pairs 72, each species 25 + 2 S; the paper's
-    forcing term instead of Guo's drops 4 + 5 + 4 x 3."""
-    f = 2 + 26 + 18 + 72 + n_species * (25 + 2 * n_species)
-    if forcing == 1:
-        f -= 4 + 5 + 12
-    return f
+def fp64_flops_per_node(n_species: int) -> int:
+    """FP64 operations of the collision of one node without a spread or body
+    force, as written (add, sub, mul and reciprocal count 1, fma 2): fluid 74,
+    each species 27 + 2 S.  The force terms (33 with Guo's forcing, 12 with the
+    paper's) run only in the warps that hold a force."""
+    return 74 + n_species * (27 + 2 * n_species)
 
 
 def max_over_ranks(x: float, dist, device) -> float:
@@ -280,8 +277,9 @@ def oracle_sample(w, target_s: float, max_steps: int, threads: int | None = None
 def run_ensemble(args, rank, world, dist):
     """64 independent tissues of uneven sizes advanced together, by one
     persistent cooperative launch per step call or by the split schedule of
-    two launches per step (either replayed from a CUDA graph; the autotuner
-    picks the schedule unless --ens-schedule names one)."""
+    two launches per step (issued one by one, the persistent one replayed
+    from a CUDA graph; the autotuner picks the schedule unless --ens-schedule
+    names one)."""
     import torch
     from paper_1503_06726_gb300 import lbib
 
@@ -368,12 +366,13 @@ def run_ensemble(args, rank, world, dist):
                    "storage": "fp32", "vertex_precision": "fp64",
                    "l2": f"inputs larger than L2: {2 * bpn * N / 2**20:.0f} MiB of populations",
                    "launch": ("split schedule: one lattice launch over every tissue and one IB "
-                              "launch over every cell per step, programmatic, one graph per "
-                              "step call" + (" (wide lattice kernel)"
+                              "launch over every cell per step, programmatic, in two groups of "
+                              "tissues from 500,000 nodes" + (" (wide lattice kernel)"
                                              if sched == lbib.LBIB_ENS_SPLIT_WIDE else "")
                               if split else "one persistent cooperative kernel per step call"),
                    "schedule": {0: "persistent", 1: "split", 2: "split_wide"}[sched],
-                   "graph": info["graph"], "grid": None if split else info["grid"],
+                   "graph": False if split else info["graph"],
+                   "grid": None if split else info["grid"],
                    "tuned": tune},
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak,
@@ -384,7 +383,10 @@ def run_ensemble(args, rank, world, dist):
                                 "of the step call)" if split else
                                 "ensemble_kernel (whole persistent launch: lattice + IB phases)"),
                      "alg_bytes_per_node": bpn, "peak_kind": f"{peak_kind} hbm_gbs (copy)"},
-        "e2e": e2e, "gpu_launches": 2 * args.steps + 1 if split else 1, "clocks": clk,
+        "e2e": e2e, "clocks": clk,
+        # two groups of tissues from half a million nodes on
+        "gpu_launches": ((2 * args.steps + 1) * (2 if N >= 500000 and len(ws) > 1 else 1)
+                         if split else 1),
         "cpu_baseline": None,
     }
 
@@ -923,7 +925,7 @@ def run_gb300(args, rank, world, dist):
         # GB300's FP64 rate, not HBM, bounds this kernel: report it against the
         # FP64 peak (nominal 1.25 TFLOP/s = 152 SMs x 2.07 GHz x 2 FP64 FMA per
         # SM per clock x 2), with the HBM figures kept beside it
-        fpn = fp64_flops_per_node(p.n_species, p.forcing)
+        fpn = fp64_flops_per_node(p.n_species)
         gflops = fpn * N / (lat_avg * 1e-3) / 1e9
         roof = dict(roof, bound="alu", achieved=gflops, peak=1250.0, unit="GFLOP/s",
                     frac=gflops / 1250.0, alg_flops_per_node=fpn,

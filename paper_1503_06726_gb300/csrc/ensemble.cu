@@ -8,9 +8,9 @@
 // lbib_ensemble_step(n) runs, for all tissues at once, the same sequence as
 // lbib_step(n): the IB prep, then per step the lattice update of every node
 // of every tissue and the IB move/prep of every cell, in the persistent kernel
-// separated by grid-wide barriers.  Work is dealt out in items -- lattice items of `nodes_per_item`
-// nodes (rows padded to 32 so a warp stays in one row) and one item per cell
-// -- strided over the persistent CTAs, which balances tissues of very
+// separated by grid-wide barriers.  Work is dealt out in items -- lattice items
+// of `nodes_per_item` nodes (rows padded to 32 so a warp stays in one row) and
+// one item per cell -- strided over the persistent CTAs, which balances tissues of very
 // different sizes.  The persistent launch is captured once per step count into
 // a CUDA graph and replayed.
 //
@@ -22,9 +22,9 @@
 // place of the grid barriers: each kernel issues its loads of what the launch
 // two back wrote before it waits on the launch just before, as the
 // single-tissue steps do.  Two groups of tissues run side by side in a large
-// ensemble.  It is the default for two tissues or more.  The schedule and the two launch parameters (nodes per item, and CTAs per SM
-// of the persistent kernel) are chosen by lbib_ensemble_tune(), which times
-// the candidates.
+// ensemble.  It is the default for two tissues or more.  The schedule and the
+// two launch parameters (nodes per item, and CTAs per SM of the persistent
+// kernel) are chosen by lbib_ensemble_tune(), which times the candidates.
 //
 // The grid barrier spins on a generation word with a bounded wait (a
 // globaltimer limit of about one second): if a barrier cannot complete, the
@@ -335,6 +335,7 @@ static EnsLatticeKernel pick_lattice_kernel(int S, int forcing, bool wide) {
 }
 
 constexpr int kEnsGroups = 2;  // groups of tissues that run side by side
+constexpr int kEnsStepsInTurn = 16;
 // nodes from which two groups are faster than one (us per step with one and
 // two: 0.39 M nodes 20.0 and 20.0, 0.57 M 24.8 and 22.2, 4.4 M 130 and 120)
 constexpr int64_t kEnsGroupNodes = 500000;
@@ -522,7 +523,9 @@ static cudaError_t ens_launch(lbib_ensemble* e, const EnsArgs& a, unsigned grid,
 // step but after the last).  Every launch after the first is programmatic;
 // without cells the lattice launches follow one another, each waiting before
 // its first load.
-static cudaError_t ens_split_group(lbib_ensemble* e, const EnsArgs& a, int g, cudaStream_t st) {
+// steps [s0, s1) of one group
+static cudaError_t ens_split_group(lbib_ensemble* e, const EnsArgs& a, int g, int s0, int s1,
+                                   cudaStream_t st) {
     const int item0 = e->group_item[g], items = e->group_item[g + 1] - item0;
     const int cell0 = e->group_cell[g], cells = e->group_cell[g + 1] - cell0;
     const size_t smem = ens_cell_smem(a.maxv);
@@ -536,8 +539,8 @@ static cudaError_t ens_split_group(lbib_ensemble* e, const EnsArgs& a, int g, cu
     };
     const EnsLatticeKernel lk =
         pick_lattice_kernel(e->S, e->forcing, e->schedule == LBIB_ENS_SPLIT_WIDE);
-    cudaError_t er = ib(0, 1, a.n_steps == 1, false);
-    for (int s = 0; s < a.n_steps && er == cudaSuccess; ++s) {
+    cudaError_t er = s0 == 0 ? ib(0, 1, a.n_steps == 1, false) : cudaSuccess;
+    for (int s = s0; s < s1 && er == cudaSuccess; ++s) {
         const bool last = (s == a.n_steps - 1);
         er = launch_kernel(lk, dim3(items), dim3(kLatticeThreads), 0, st, cells > 0 || s > 0, a, s,
                            last ? 1 : 0, item0);
@@ -566,10 +569,13 @@ static cudaError_t ens_split_enqueue(lbib_ensemble* e, const EnsArgs& a, cudaStr
             er = cudaEventCreateWithFlags(&e->join[g], cudaEventDisableTiming);
         if (er == cudaSuccess) er = cudaStreamWaitEvent(e->branch[g], e->fork, 0);
     }
-    // (both groups' launches in turn would keep the host nearer to both
-    // streams; a group's launches are a few microseconds each, its steps tens)
-    for (int g = 0; g < groups && er == cudaSuccess; ++g)
-        er = ens_split_group(e, a, g, g ? e->branch[g] : st);
+    // a few steps of each group in turn: a stream takes about a thousand
+    // launches before it makes the host wait, which with one group's steps
+    // first would leave the other group waiting too
+    for (int s = 0; s < a.n_steps && er == cudaSuccess; s += kEnsStepsInTurn)
+        for (int g = 0; g < groups && er == cudaSuccess; ++g)
+            er = ens_split_group(e, a, g, s, std::min(a.n_steps, s + kEnsStepsInTurn),
+                                 g ? e->branch[g] : st);
     // whatever was enqueued on the branches ends before the stream goes on
     for (int g = 1; g < groups && e->join[g]; ++g) {
         const cudaError_t e1 = cudaEventRecord(e->join[g], e->branch[g]);

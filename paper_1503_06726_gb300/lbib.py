@@ -590,10 +590,11 @@ def _ens_check(rc, ens):
 
 
 class Ensemble:
-    """Many independent FP32 tissues advanced by one persistent launch per
-    step call, or by two launches per step (the split schedules).  ``params``
-    is a list of parameter objects; ``tissues`` the matching list of tissues
-    (lbib_inputs.Tissue-like; None for a tissue without cells)."""
+    """Many independent FP32 tissues advanced by two launches per step (the
+    split schedules, the default of several tissues), or by one persistent
+    launch per step call.  ``params`` is a list of parameter objects;
+    ``tissues`` the matching list of tissues (lbib_inputs.Tissue-like; None for
+    a tissue without cells)."""
 
     def __init__(self, params, tissues, device=None, stream=None):
         import torch
