@@ -583,8 +583,9 @@ __global__ void tile_weights_tc_kernel(const __nv_bfloat16* w, int Co, int Ci, i
 // three (256^2, 16 images: 32 -> 32 channels 75 us with one row at a time, 61
 // with three; 80 -> 32 251 and 189).  Where 3 Np exceeds the largest N of 256,
 // the first two or one, then the others (the network's levels of 32^2 and 16^2:
-// 19 us, and 18 with one row at a time and no halo of G).  The K steps walk the tile's image rows 16 pixels at a time (Wt a
-// multiple of 16), so the halo columns never enter.  One accumulator per
+// 19 us, and 18 with one row at a time and no halo of G).  The K steps walk the
+// tile's image rows 16 pixels at a time (Wt a multiple of 16), so the halo
+// columns never enter.  One accumulator per
 // "set" of image rows (rows r % sets; more independent accumulation chains in
 // flight), summed at the end and added to dW with FP32 reductions.  A CTA
 // takes one input-channel chunk, one N tile and a range of pixel tiles

@@ -5,14 +5,15 @@
 // channel counts multiples of 16.
 //
 // Convolution as an implicit GEMM: M = output pixels (a CTA tile of 8 x 16
-// pixels of one image), N = output channels (64 per CTA), K = 9 taps x input
-// channels (chunks of 32).  Per K chunk the CTA stages the 10 x 18 halo of
-// its pixel tile and the weights of all 9 taps in shared memory with
-// cp.async (zero fill outside the image), then every warp multiplies its
-// 32 x 32 block with mma.sync m16n8k16 (BF16 in, FP32 accumulate) fed by
-// ldmatrix.  The input may be the concatenation [x1, upsample2(x2)] of a
-// full-resolution tensor and a half-resolution one; the upsampling is done
-// while loading, so the decoder never materialises the concatenation.
+// pixels of one image), N = output channels (64 per CTA, 32 where the grid is
+// small), K = 9 taps x input channels (chunks of 32).  Per K chunk the CTA
+// stages the 10 x 18 halo of its pixel tile and the weights of all 9 taps in
+// shared memory with cp.async (zero fill outside the image), then every warp
+// multiplies its 32 x 32 block with mma.sync m16n8k16 (BF16 in, FP32
+// accumulate) fed by ldmatrix.  The input may be the concatenation [x1,
+// upsample2(x2)] of a full-resolution tensor and a half-resolution one; the
+// upsampling is done while loading, so the decoder never materialises the
+// concatenation.
 #include <cuda_bf16.h>
 
 #include <cstdint>
